@@ -503,7 +503,7 @@ struct claw_solver {
   int npart = 0;
   int ntiles = 0, bw = 128, h = 32;
   int tuned = 0;
-  void* work3 = nullptr;  // 3D per-face arrays
+  void* work3 = nullptr;  // per-face path: face arrays
   size_t work3_bytes = 0;
   cudaGraphExec_t gexec = nullptr;
   int gk = 0;
@@ -546,7 +546,7 @@ cudaError_t leave(claw_solver* s) {
 cudaError_t solver_attempt(claw_solver* s, cudaStream_t st) {
   if (s->nd == 3) {
     LaunchArgs a{s->d_mem, nullptr, s->ntiles, s->consts.data(), 0, 0, 0, st,
-                 {(int)s->g.n[0], (int)s->g.n[1], (int)s->g.n[2]}, s->work3, s->work3_bytes};
+                 {(int)s->g.n[0], (int)s->g.n[1], (int)s->g.n[2]}, nullptr, 0};
     return s->ks.classic(a);
   }
   const int n3[3] = {(int)s->g.n[0], (int)s->g.n[1], (int)s->g.n[2]};
@@ -813,7 +813,7 @@ claw_status claw_solver_create(const claw_method* m, const claw_grid* g, void* s
                  ? 1
                  : 0;
   if (s->faces) s->tuned = 1;  // no tile shapes to choose
-  s->ntiles = s->nd == 3 ? classic3d_update_blocks(cells_of(s->g))
+  s->ntiles = s->nd == 3 ? ks.blocks3((int)s->g.n[0], (int)s->g.n[1], (int)s->g.n[2])
              : s->faces    ? (int)((cells_of(s->g) + 255) / 256)
                            : tiles_of(m->scheme, s->nd, s->prec, s->ks.MA, (int)s->g.n[0],
                              (int)s->g.n[1], s->bw, s->h);
@@ -833,11 +833,6 @@ claw_status claw_bind_state(claw_solver* s, void* q_dev, const void* aux_dev, do
   if (s->faces) {
     s->work3_bytes = faces_work_bytes(s->nd, (int)s->g.n[0], (int)s->g.n[1], s->m.num_eqn,
                                       s->prec);
-    SCK(cudaMalloc(&s->work3, s->work3_bytes));
-  }
-  if (s->nd == 3) {
-    s->work3_bytes = classic3d_work_bytes((int)s->g.n[0], (int)s->g.n[1], (int)s->g.n[2],
-                                          s->m.num_eqn, s->prec);
     SCK(cudaMalloc(&s->work3, s->work3_bytes));
   }
   SCK(cudaMalloc(&s->d_ctl, sizeof(DevCtl)));
@@ -1216,12 +1211,12 @@ void batch_free(claw_batch* b) {
 
 cudaError_t batch_attempt(claw_batch* b, cudaStream_t st) {
   if (b->nd == 3) {
-    // sweeps and update of one 3D member at a time, each on its own face arrays
+    // one 3D member at a time
     cudaError_t e = cudaSuccess;
     for (int k = 0; k < b->n && e == cudaSuccess; ++k) {
       const Member& mb = b->h_mem[k];
       LaunchArgs a{b->d_mem + k, nullptr, mb.ntiles, b->consts.data(), 0, 0, 0, st,
-                   {mb.nx, mb.ny, mb.nz}, mb.work3, b->work3_bytes[k]};
+                   {mb.nx, mb.ny, mb.nz}, nullptr, 0};
       e = b->ks.classic(a);
     }
     return e;
@@ -1300,17 +1295,6 @@ claw_status claw_batch_bind(claw_batch* b, void* const* q, const void* const* au
     total += b->sbytes[k] * (b->nbuf - 1 + pre_buffers(b->m));
   }
   BCK(cudaMalloc(&b->work, total));
-  if (b->nd == 3) {
-    size_t w3 = 0;
-    b->work3_bytes.assign(n, 0);
-    for (int k = 0; k < n; ++k) {
-      const claw_grid& g = b->grids[k];
-      b->work3_bytes[k] = align256(classic3d_work_bytes((int)g.n[0], (int)g.n[1], (int)g.n[2],
-                                                        b->m.num_eqn, b->prec));
-      w3 += b->work3_bytes[k];
-    }
-    BCK(cudaMalloc(&b->work3, w3));
-  }
   if (b->faces) {
     size_t w3 = 0;
     b->work3_bytes.assign(n, 0);
@@ -1358,11 +1342,9 @@ claw_status claw_batch_bind(claw_batch* b, void* const* q, const void* const* au
     mb.nz = 1;
     mb.ctl = b->d_ctl + k;
     if (b->nd == 3) {
-      // the 3D kernels take one member; the update's blocks count the arrivals
+      // the 3D kernel takes one member; its blocks count the arrivals
       mb.nz = (int)g.n[2];
-      mb.ntiles = classic3d_update_blocks(cells_of(g));
-      mb.work3 = w3p;
-      w3p += b->work3_bytes[k];
+      mb.ntiles = b->ks.blocks3(mb.nx, mb.ny, mb.nz);
     } else if (b->faces) {
       // the update's blocks (256 cells each) count the arrivals
       mb.ntiles = (int)((cells_of(g) + 255) / 256);
@@ -1655,9 +1637,6 @@ claw_status sfail(claw_server* v, const char* what, cudaError_t e = cudaSuccess)
   } while (0)
 
 size_t req_faces_bytes(const claw_server* v, const claw_grid& g) {
-  if (v->nd == 3)
-    return align256(classic3d_work_bytes((int)g.n[0], (int)g.n[1], (int)g.n[2], v->m.num_eqn,
-                                         v->prec));
   return v->faces ? align256(faces_work_bytes(v->nd, (int)g.n[0], (int)g.n[1], v->m.num_eqn,
                                               v->prec))
                   : 0;
@@ -1798,11 +1777,11 @@ claw_status claw_server_pump(claw_server* v, int steps, int* running, int* queue
   if (!v->sel.empty()) {
     for (int i = 0; i < steps; ++i) {
       if (v->nd == 3) {
-        // the 3D sweeps take one member: request by request
+        // the 3D kernel takes one member: request by request
         for (size_t k = 0; k < v->sel.size(); ++k) {
           const Req& r = v->reqs[v->sel[k]];
           LaunchArgs a{v->d_smem + k, nullptr, r.mem.ntiles, v->consts.data(), 0, 0, 0, v->st,
-                       {r.mem.nx, r.mem.ny, r.mem.nz}, r.mem.work3, r.w3bytes};
+                       {r.mem.nx, r.mem.ny, r.mem.nz}, nullptr, 0};
           VCK(v->ks.classic(a));
         }
       } else if (v->faces) {
@@ -1902,12 +1881,13 @@ claw_status claw_server_pump(claw_server* v, int steps, int* running, int* queue
     r.mem.nx = (int)r.g.n[0];
     r.mem.ny = (int)r.g.n[1];
     r.mem.nz = v->nd == 3 ? (int)r.g.n[2] : 1;
-    if (v->faces || v->nd == 3) {
+    if (v->faces) {
       // face arrays; the update's blocks (256 cells each) count the arrivals
       r.w3bytes = req_faces_bytes(v, r.g);
       r.mem.work3 = p;
-      r.mem.ntiles = v->nd == 3 ? classic3d_update_blocks(cells_of(r.g))
-                                : (int)((cells_of(r.g) + 255) / 256);
+      r.mem.ntiles = (int)((cells_of(r.g) + 255) / 256);
+    } else if (v->nd == 3) {
+      r.mem.ntiles = v->ks.blocks3(r.mem.nx, r.mem.ny, r.mem.nz);
     } else {
       r.mem.ntiles =
           tiles_of(v->m.scheme, v->nd, v->prec, v->ks.MA, r.mem.nx, r.mem.ny, v->bw, v->h);

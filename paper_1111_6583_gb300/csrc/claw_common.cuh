@@ -56,7 +56,7 @@ struct Member {
   int ntiles;        // blocks of this member per attempt
   int nz;            // 3D: cells in z (1 otherwise)
   DevCtl* ctl;
-  void* work3;       // 3D: per-face fluctuation / correction arrays
+  void* work3;       // per-face path: face records
   void* qpre;        // Strang-split source: Q^n after the first half source
                      // step, which the step reads in place of slot cur; else null
 };

@@ -27,8 +27,8 @@ struct LaunchArgs {
                            // work (kWork1dTiles, kWork1dUnits, else automatic)
   int stage;               // SharpClaw SSP-RK3 stage 0..2 (used when stage_op is null)
   cudaStream_t stream;
-  int n3[3];               // 3D: cells per direction
-  void* work3;             // 3D: per-face arrays (device)
+  int n3[3];               // 3D and the per-face path: cells per direction
+  void* work3;             // per-face path: face arrays (device)
   size_t work3_bytes;
   const StageOp* stage_op; // SharpClaw: explicit stage (host pointer) or null
   int sweep;               // 2D classic: 0 unsplit, 1 / 2 the x / y sweeps of a split step
@@ -52,6 +52,7 @@ struct KernelSet {
   launch_fn maxspeed;      // first-order interface speeds into ctl->smax
   launch_fn source;        // axisymmetric Euler source step (2D Euler systems)
   int max_bw;              // 2D classic: widest block whose static shared memory fits
+  int (*blocks3)(int nx, int ny, int nz);  // 3D: blocks of an attempt (they count the arrivals)
   int sharp_shapes;        // 2D SharpClaw WENO5: bit i set when tile kSharpShapes2[i]
                            // fits in a block's shared memory
 };
@@ -124,18 +125,6 @@ __host__ __device__ inline int classic2d_tiles(int nx, int ny, int BW, int H) {
 }
 __host__ __device__ inline int sharp_tiles(int nx, int ny, int TX, int TY) {
   return ((nx + TX - 1) / TX) * ((ny + TY - 1) / TY);
-}
-
-// 3D update: cells per block (256 threads, four cells each); the update's
-// blocks count the arrivals for the controller
-constexpr int kUpdateCells3d = 1024;
-inline int classic3d_update_blocks(long long cells) {
-  return (int)((cells + kUpdateCells3d - 1) / kUpdateCells3d);
-}
-
-inline size_t classic3d_work_bytes(int nx, int ny, int nz, int M, int prec) {
-  size_t faces = (size_t)(nx + 1) * ny * nz + (size_t)nx * (ny + 1) * nz + (size_t)nx * ny * (nz + 1);
-  return faces * 3 * M * (prec == 0 ? 8 : 4);
 }
 
 KernelSet claw_kernels_advection(int nd, int prec);

@@ -200,27 +200,12 @@ struct Launchers {
     }
     if constexpr (ND == 3) {
       const long long nx = a.n3[0], ny = a.n3[1], nz = a.n3[2];
-      // with transverse terms the x sweep writes every record first (no fill)
-      if (!C.transverse) {
-        cudaError_t e = cudaMemsetAsync(a.work3, 0, a.work3_bytes, a.stream);
-        if (e != cudaSuccess) return e;
-      }
-      // x: lanes along x, a block of kXSweepLines y lines walks a segment of
-      // z planes; y, z: one block per patch of lines and segment of cells
-      // along the sweep
-      constexpr int NW = kXSweepLines, NB = sizeof(R) == 4 ? 2 : 1;
-      int nxc, nyb, nzs;
-      xsweep3d_grid(NW, (int)nx, (int)ny, (int)nz, nxc, nyb, nzs);
-      classic3d_xsweep<RP, R, NW, NB><<<(unsigned)(nxc * nyb * nzs), 32 * NW, 0, a.stream>>>(
-          a.members, C);
-      int npf, nps, nseg;
-      sweep3d_grid(1, (int)nx, (int)ny, (int)nz, npf, nps, nseg);
-      classic3d_sweep<RP, R, 1><<<(unsigned)(npf * nps * nseg), kPatch3d * kPatch3d, 0,
-                                  a.stream>>>(a.members, C);
-      sweep3d_grid(2, (int)nx, (int)ny, (int)nz, npf, nps, nseg);
-      classic3d_sweep<RP, R, 2><<<(unsigned)(npf * nps * nseg), kPatch3d * kPatch3d, 0,
-                                  a.stream>>>(a.members, C);
-      classic3d_update<RP, R><<<a.ntiles_total, 256, 0, a.stream>>>(a.members, C);
+      const Layout3 L = layout3d((int)nx, (int)ny, (int)nz, sizeof(R) == 8 ? 0 : 1);
+      const unsigned grid = (unsigned)classic3d_blocks(L);
+      if (C.lim == CLAW_LIM_MC && C.order == 2 && C.transverse == 2)
+        classic3d_kernel<RP, R, true><<<grid, 32 * kXSweepLines, 0, a.stream>>>(a.members, C, L);
+      else
+        classic3d_kernel<RP, R, false><<<grid, 32 * kXSweepLines, 0, a.stream>>>(a.members, C, L);
       return cudaGetLastError();
     } else if constexpr (ND == 2 && RP::MA > 0) {
       // 2D solvers with aux fields have normal solves only (SharpClaw)
@@ -386,6 +371,9 @@ struct Launchers {
       return cudaErrorNotSupported;
     }
   }
+  static int blocks3(int nx, int ny, int nz) {
+    return classic3d_blocks(layout3d(nx, ny, nz, sizeof(R) == 8 ? 0 : 1));
+  }
   static cudaError_t maxspeed(const LaunchArgs& a) {
     const MConsts<R>& C = *(const MConsts<R>*)a.consts;
     if constexpr (ND == 3) {
@@ -412,6 +400,7 @@ KernelSet make_set(bool has_char) {
   k.sharp = &Launchers<RP, R, ND>::sharp;
   k.maxspeed = &Launchers<RP, R, ND>::maxspeed;
   k.source = &Launchers<RP, R, ND>::source;
+  k.blocks3 = &Launchers<RP, R, ND>::blocks3;
   k.max_bw = classic2d_fits<RP, R>(128) ? 128 : 64;
   constexpr size_t lim = kSmemPerBlock;
   k.sharp_shapes = (sharp_smem_bytes<RP, R, 2, 16, 8, 3>() <= lim ? 1 : 0) |
