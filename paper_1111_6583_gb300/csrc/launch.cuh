@@ -6,6 +6,7 @@
 #include "classic3d.cuh"
 #include "classic_faces.cuh"
 #include "kernels.h"
+#include "linear2d.cuh"
 #include "sharpclaw.cuh"
 
 namespace claw {
@@ -219,8 +220,8 @@ struct Launchers {
       // systems of up to three fields: with more, the two block widths of the
       // fixed-settings form were seen to round differently, and every tile
       // shape must give the same bits
-      if (sizeof(R) == 4 && RP::M <= 3 && C.lim == CLAW_LIM_MC && C.order == 2 &&
-          C.transverse == 2)
+      if ((sizeof(R) == 4 || is_linear_rp<RP, R>::value) && RP::M <= 3 && C.lim == CLAW_LIM_MC && C.order == 2 &&
+          C.transverse == 2 && a.sweep == 0)
         return classic2d<true>(a, C);
       return classic2d<false>(a, C);
     }
@@ -270,7 +271,17 @@ struct Launchers {
   }
   template <bool FAST>
   static cudaError_t classic2d(const LaunchArgs& a, const MConsts<R>& C) {
-    if constexpr (ND == 2 && RP::MA == 0 && (!FAST || (sizeof(R) == 4 && RP::M <= 3))) {
+    if constexpr (ND == 2 && is_linear_rp<RP, R>::value) {
+      // bits do not depend on FAST or on the width (explicit rounding)
+      const unsigned grid = (unsigned)launch_grid(a.ntiles_total);
+      if (a.bw == 128)
+        linear2d_kernel<RP, R, 128, FAST><<<grid, 32, 0, a.stream>>>(a.members, a.tiles, C, a.h, a.sweep);
+      else if (a.bw == 64)
+        linear2d_kernel<RP, R, 64, FAST><<<grid, 32, 0, a.stream>>>(a.members, a.tiles, C, a.h, a.sweep);
+      else
+        return cudaErrorInvalidValue;
+      return cudaGetLastError();
+    } else if constexpr (ND == 2 && RP::MA == 0 && (!FAST || (sizeof(R) == 4 && RP::M <= 3))) {
       if constexpr (classic2d_fits<RP, R>(128)) {
         if (a.bw == 128) {
           classic2d_kernel<RP, R, 128, FAST><<<launch_grid(a.ntiles_total), 128, 0, a.stream>>>(
