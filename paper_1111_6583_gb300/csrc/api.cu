@@ -182,10 +182,19 @@ const char* check_grid(const claw_grid& g, const claw_method& m) {
   return nullptr;
 }
 
-// ma: the solver's aux fields (the 1D classic tile depends on them)
-int tiles_of(int scheme, int nd, int prec, int ma, int nx, int ny, int bw, int h) {
+// the classic step runs on the per-face path (a capacity; 2D acoustics in a
+// varying medium has its own kernel, capacity included)
+int on_faces(const claw_method& m, int nd) {
+  return m.scheme == CLAW_CLASSIC && nd <= 2 && m.capa_index >= 0 &&
+                 !(nd == 2 && m.rp == CLAW_RP_ACOUSTICS_VC)
+             ? 1
+             : 0;
+}
+
+int tiles_of(const KernelSet& ks, int scheme, int nd, int prec, int nx, int ny, int bw, int h) {
   if (scheme == CLAW_CLASSIC)
-    return nd == 1 ? classic1d_tiles(nx, prec, ma) : classic2d_tiles(nx, ny, bw, h);
+    return nd == 1 ? classic1d_tiles(nx, prec, ks.MA)
+                   : classic2d_tiles(nx, ny, bw == 64 ? ks.tx64 : ks.tx128, h);
   if (nd == 1) return sharp_tiles(nx, 1, kSharpTX1, 1);
   int tx, ty;
   sharp2d_shape(bw, h, tx, ty);
@@ -293,7 +302,7 @@ cudaError_t tune_members(const KernelSet& ks, int nd, const claw_method& m,
     if (e != cudaSuccess) break;
     std::vector<Tile> tt;
     for (int k = 0; k < n; ++k) {
-      tm[k].ntiles = tiles_of(m.scheme, nd, m.prec, ks.MA, tm[k].nx, tm[k].ny, pr.first,
+      tm[k].ntiles = tiles_of(ks, m.scheme, nd, m.prec, tm[k].nx, tm[k].ny, pr.first,
                               pr.second);
       for (int t = 0; t < tm[k].ntiles; ++t) tt.push_back(Tile{k, t});
     }
@@ -483,7 +492,7 @@ struct claw_solver {
   claw_method m;
   claw_grid g;
   int nd = 1, prec = 0, nbuf = 2;
-  int faces = 0;  // classic step on the per-face path (capacity / media-aware transverse)
+  int faces = 0;  // classic step on the per-face path (capacity)
   KernelSet ks{};
   std::vector<unsigned char> consts;
   cudaStream_t ustream = nullptr, st = nullptr;
@@ -611,7 +620,7 @@ cudaError_t autotune(claw_solver* s) {
     if (e != cudaSuccess) return e;
     s->bw = bw;
     s->h = h;
-    s->ntiles = tiles_of(s->m.scheme, 2, s->prec, s->ks.MA, (int)s->g.n[0], (int)s->g.n[1],
+    s->ntiles = tiles_of(s->ks, s->m.scheme, 2, s->prec, (int)s->g.n[0], (int)s->g.n[1],
                          bw, h);
     s->tuned = 1;
     drop_graph(s);
@@ -648,8 +657,8 @@ cudaError_t autotune(claw_solver* s) {
       if (h <= 2 * ny) cand.push_back({bw, h});
     for (int k = 1; k <= 8; ++k) {
       if (nsm <= 0) break;
-      int h = 4;
-      while (h < ny && classic2d_tiles(nx, ny, bw, h) > k * nsm) ++h;
+      int h = s->ks.reg_kernel ? 2 : 4;
+      while (h < ny && tiles_of(s->ks, s->m.scheme, 2, s->prec, nx, ny, bw, h) > k * nsm) ++h;
       bool seen = false;
       for (auto& pr : cand) seen |= (pr.first == bw && pr.second == h);
       if (!seen) cand.push_back({bw, h});
@@ -662,7 +671,7 @@ cudaError_t autotune(claw_solver* s) {
   int bb = s->ks.max_bw, bh = 32;
   for (const auto& pr : cand) {
     const int bw = pr.first, h = pr.second;
-    const int nt = classic2d_tiles(nx, ny, bw, h);
+    const int nt = tiles_of(s->ks, s->m.scheme, 2, s->prec, nx, ny, bw, h);
     mt.ntiles = nt;
     if ((e = cudaMemcpyAsync(s->d_mem_tune, &mt, sizeof(Member), cudaMemcpyHostToDevice,
                              s->st)) != cudaSuccess)
@@ -686,7 +695,7 @@ cudaError_t autotune(claw_solver* s) {
   if (e != cudaSuccess) return e;
   s->bw = bb;
   s->h = bh;
-  s->ntiles = classic2d_tiles(nx, ny, bb, bh);
+  s->ntiles = tiles_of(s->ks, s->m.scheme, 2, s->prec, nx, ny, bb, bh);
   s->tuned = 1;
   drop_graph(s);
   return upload_member(s);
@@ -808,14 +817,11 @@ claw_status claw_solver_create(const claw_method* m, const claw_grid* g, void* s
     claw_solver_destroy(s);
     return st;
   }
-  s->faces = (m->scheme == CLAW_CLASSIC && s->nd <= 2 &&
-              (m->capa_index >= 0 || (s->nd == 2 && m->rp == CLAW_RP_ACOUSTICS_VC)))
-                 ? 1
-                 : 0;
+  s->faces = on_faces(*m, s->nd);
   if (s->faces) s->tuned = 1;  // no tile shapes to choose
   s->ntiles = s->nd == 3 ? ks.blocks3((int)s->g.n[0], (int)s->g.n[1], (int)s->g.n[2])
              : s->faces    ? (int)((cells_of(s->g) + 255) / 256)
-                           : tiles_of(m->scheme, s->nd, s->prec, s->ks.MA, (int)s->g.n[0],
+                           : tiles_of(s->ks, m->scheme, s->nd, s->prec, (int)s->g.n[0],
                              (int)s->g.n[1], s->bw, s->h);
   *out = s;
   return CLAW_OK;
@@ -890,7 +896,7 @@ claw_status claw_solver_tune(claw_solver* s, int mode, int* bw, int* h) {
     s->bw = *bw;
     s->h = *h;
     if (s->nd != 3 && !s->faces)
-      s->ntiles = tiles_of(s->m.scheme, s->nd, s->prec, s->ks.MA, (int)s->g.n[0],
+      s->ntiles = tiles_of(s->ks, s->m.scheme, s->nd, s->prec, (int)s->g.n[0],
                            (int)s->g.n[1], s->bw, s->h);
     s->tuned = 1;
     drop_graph(s);
@@ -1153,7 +1159,7 @@ struct claw_batch {
   int* d_count = nullptr;
   int* h_count = nullptr;
   int bw = 128, h = 32;
-  int faces = 0;              // per-face classic path (capacity / media-aware transverse)
+  int faces = 0;              // per-face classic path (capacity)
   void* work3 = nullptr;      // the members' face arrays, one allocation
   std::vector<size_t> work3_bytes;
   Tile* d_tile0 = nullptr;    // (member 0, t) for the source steps of one member at a time
@@ -1246,8 +1252,7 @@ claw_status claw_batch_create(const claw_method* m, const claw_grid* grids, int 
   if (!m || !grids || !out || n <= 0) return bfail(nullptr, "bad argument");
   *out = nullptr;
   const int nd = grids[0].ndim;
-  const int faces = m->scheme == CLAW_CLASSIC && nd <= 2 &&
-                    (m->capa_index >= 0 || (nd == 2 && m->rp == CLAW_RP_ACOUSTICS_VC));
+  const int faces = on_faces(*m, nd);
   for (int k = 0; k < n; ++k) {
     if (const char* why = check_grid(grids[k], *m)) return bfail(nullptr, why);
     if (grids[k].ndim != nd) return bfail(nullptr, "all members need the same ndim");
@@ -1351,7 +1356,7 @@ claw_status claw_batch_bind(claw_batch* b, void* const* q, const void* const* au
       mb.work3 = w3p;
       w3p += b->work3_bytes[k];
     } else {
-      mb.ntiles = tiles_of(b->m.scheme, b->nd, b->prec, b->ks.MA, mb.nx, mb.ny, b->bw, b->h);
+      mb.ntiles = tiles_of(b->ks, b->m.scheme, b->nd, b->prec, mb.nx, mb.ny, b->bw, b->h);
       for (int t = 0; t < mb.ntiles; ++t) b->h_tiles.push_back(Tile{k, t});
     }
     const int ms = b->nd == 3 ? 0 : maxspeed_tiles(mb.nx, mb.ny);
@@ -1509,7 +1514,7 @@ claw_status claw_batch_tune(claw_batch* b, int mode, int* bw, int* h) {
     b->h_tiles.clear();
     for (int k = 0; k < b->n; ++k) {
       Member& mb = b->h_mem[k];
-      mb.ntiles = tiles_of(b->m.scheme, b->nd, b->prec, b->ks.MA, mb.nx, mb.ny, b->bw, b->h);
+      mb.ntiles = tiles_of(b->ks, b->m.scheme, b->nd, b->prec, mb.nx, mb.ny, b->bw, b->h);
       for (int t = 0; t < mb.ntiles; ++t) b->h_tiles.push_back(Tile{k, t});
     }
     if ((int)b->h_tiles.size() > b->ntiles) {
@@ -1659,8 +1664,7 @@ claw_status claw_server_create_nd(const claw_method* m, int ndim, size_t hbm_bud
   *out = nullptr;
   const int nd = ndim;
   if (const char* why = check_method(*m, nd)) return sfail(nullptr, why);
-  const int faces = m->scheme == CLAW_CLASSIC && nd <= 2 &&
-                    (m->capa_index >= 0 || (nd == 2 && m->rp == CLAW_RP_ACOUSTICS_VC));
+  const int faces = on_faces(*m, nd);
   KernelSet ks = kernels_for(m->rp, nd, m->prec);
   if (!ks.valid) return sfail(nullptr, "no kernels for this solver/dimension/precision");
   claw_server* v = new claw_server();
@@ -1890,7 +1894,7 @@ claw_status claw_server_pump(claw_server* v, int steps, int* running, int* queue
       r.mem.ntiles = v->ks.blocks3(r.mem.nx, r.mem.ny, r.mem.nz);
     } else {
       r.mem.ntiles =
-          tiles_of(v->m.scheme, v->nd, v->prec, v->ks.MA, r.mem.nx, r.mem.ny, v->bw, v->h);
+          tiles_of(v->ks, v->m.scheme, v->nd, v->prec, r.mem.nx, r.mem.ny, v->bw, v->h);
     }
     DevCtl c = make_ctl(v->m, r.g, v->nbuf, 0.0, r.t_end);
     VCK(stage_upload(v, r.mem.q[0], r.q0.data(), r.q0.size()));
@@ -2119,7 +2123,7 @@ claw_status claw_server_tune(claw_server* v, int mode, int* bw, int* h) {
     // running requests take the new shape from their next attempt on
     for (uint64_t t : v->running) {
       Req& r = v->reqs[t];
-      r.mem.ntiles = tiles_of(v->m.scheme, v->nd, v->prec, v->ks.MA, r.mem.nx, r.mem.ny, v->bw,
+      r.mem.ntiles = tiles_of(v->ks, v->m.scheme, v->nd, v->prec, r.mem.nx, r.mem.ny, v->bw,
                               v->h);
     }
     v->sel.clear();

@@ -697,7 +697,7 @@ __global__ void __launch_bounds__(BW)
       continue;
     }
     const int nx = mb.nx, ny = mb.ny;
-    const Classic2dLayout L = classic2d_layout(nx, ny, BW, H);
+    const Classic2dLayout L = classic2d_layout(nx, ny, TX, H);
     const int c0 = (tl.tile % L.nsx) * TX;
     const int ch = tl.tile / L.nsx;
     const int r0 = (int)(((long long)ch * ny) / L.nch);

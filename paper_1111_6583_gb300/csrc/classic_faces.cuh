@@ -1,8 +1,7 @@
 // classic_faces.cuh -- the classic step (Sec. 2, Eq. (fluxdiff), Eq. (lwflux);
 // Sec. 2.1 transverse propagation) on a per-face decomposition, for the cases
 // the row-walk kernels do not cover: a capacity function kappa (Eq. (conslaw),
-// capacity-form differencing) in 1D or 2D, and 2D solvers whose transverse
-// split needs the media of the neighbouring cells.
+// capacity-form differencing) in 1D or 2D.
 //
 // One attempt = a sweep per direction that writes a record per face (y
 // faces: a thread per face loads the four cells of the face's limiter
@@ -170,26 +169,8 @@ __global__ void __launch_bounds__(kFacesThreads)
         tp[k] = C.transverse == 2 ? ap[k] - F[k] : ap[k];
         tm[k] = C.transverse == 2 ? am[k] + F[k] : am[k];
       }
-      if constexpr (trans_aux_rp<RP>::value) {
-        // media of the transverse neighbours of the two cells
-        R mr[MAS], pr[MAS], ml[MAS], pl[MAS];
-        if (D == 0) {
-          load_aux<MA, R>(C, aux, nx, ny, f, l - 1, mr);
-          load_aux<MA, R>(C, aux, nx, ny, f, l + 1, pr);
-          load_aux<MA, R>(C, aux, nx, ny, f - 1, l - 1, ml);
-          load_aux<MA, R>(C, aux, nx, ny, f - 1, l + 1, pl);
-        } else {
-          load_aux<MA, R>(C, aux, nx, ny, l - 1, f, mr);
-          load_aux<MA, R>(C, aux, nx, ny, l + 1, f, pr);
-          load_aux<MA, R>(C, aux, nx, ny, l - 1, f - 1, ml);
-          load_aux<MA, R>(C, aux, nx, ny, l + 1, f - 1, pl);
-        }
-        RP::template trans_aux<D>(C, mr, au[2], pr, tp, bma, bpa);
-        RP::template trans_aux<D>(C, ml, au[1], pl, tm, bmb, bpb);
-      } else {
-        RP::template trans<D>(C, x, tp, bma, bpa);
-        RP::template trans<D>(C, x, tm, bmb, bpb);
-      }
+      RP::template trans<D>(C, x, tp, bma, bpa);
+      RP::template trans<D>(C, x, tm, bmb, bpb);
       if (C.capa >= 0) {
 #pragma unroll
         for (int k = 0; k < M; ++k) {

@@ -52,6 +52,8 @@ struct KernelSet {
   launch_fn maxspeed;      // first-order interface speeds into ctl->smax
   launch_fn source;        // axisymmetric Euler source step (2D Euler systems)
   int max_bw;              // 2D classic: widest block whose static shared memory fits
+  int tx64, tx128;         // 2D classic: columns of a tile at either width
+  int reg_kernel;          // 2D classic: register-resident kernel (chunks of 2 rows pay)
   int (*blocks3)(int nx, int ny, int nz);  // 3D: blocks of an attempt (they count the arrivals)
   int sharp_shapes;        // 2D SharpClaw WENO5: bit i set when tile kSharpShapes2[i]
                            // fits in a block's shared memory
@@ -102,8 +104,9 @@ inline void sharp2d_shape(int bw, int h, int& tx, int& ty) {
 }
 constexpr int kMaxspeedCells = 256;           // cells per max-speed block
 
-// Tiles of the 2D classic kernel.  A block of BW threads owns a strip of
-// TX = BW - 4 interior columns and a chunk of rows; the ny rows are spread
+// Tiles of the 2D classic kernels.  A block owns a strip of TX interior
+// columns (BW - 4 for a block of BW threads; reg_tile for the
+// register-resident kernels) and a chunk of rows; the ny rows are spread
 // evenly over nch = ceil(ny / H) chunks (no short last chunk).  Tile t is
 // strip t % nsx, chunk t / nsx.  In a narrow last strip the warps that hold
 // only columns past the second ghost column skip all work; its chunks keep
@@ -112,16 +115,29 @@ constexpr int kMaxspeedCells = 256;           // cells per max-speed block
 struct Classic2dLayout {
   int TX, nsx, nch;
 };
-__host__ __device__ inline Classic2dLayout classic2d_layout(int nx, int ny, int BW, int H) {
+__host__ __device__ inline Classic2dLayout classic2d_layout(int nx, int ny, int TX, int H) {
   Classic2dLayout L;
-  L.TX = BW - 4;
+  L.TX = TX;
   L.nsx = (nx + L.TX - 1) / L.TX;
   L.nch = (ny + H - 1) / H;
   return L;
 }
-__host__ __device__ inline int classic2d_tiles(int nx, int ny, int BW, int H) {
-  const Classic2dLayout L = classic2d_layout(nx, ny, BW, H);
+__host__ __device__ inline int classic2d_tiles(int nx, int ny, int TX, int H) {
+  const Classic2dLayout L = classic2d_layout(nx, ny, TX, H);
   return L.nsx * L.nch;
+}
+// The register-resident 2D kernels (linear2d.cuh, medium2d.cuh): columns per
+// lane, warps per block (side by side, each with its own halo) and columns of
+// a tile for the launch width BW.  FP64: a warp's FP64 instruction holds its
+// sub-partition's unit for 64 cycles, so small grids want many narrow warps
+// (one column per lane; acoustics 64^2 47 -> 28 us/step against two) and two
+// columns are the widest that fit the registers; FP32: two or four columns.
+struct RegTile {
+  int n, warps, tx;
+};
+__host__ __device__ constexpr RegTile reg_tile(int prec, int bw) {
+  return prec == 0 ? RegTile{bw == 128 ? 2 : 1, 2, bw == 128 ? 120 : 56}
+                   : RegTile{bw == 128 ? 4 : 2, 1, bw == 128 ? 124 : 60};
 }
 __host__ __device__ inline int sharp_tiles(int nx, int ny, int TX, int TY) {
   return ((nx + TX - 1) / TX) * ((ny + TY - 1) / TY);

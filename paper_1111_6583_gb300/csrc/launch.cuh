@@ -7,6 +7,7 @@
 #include "classic_faces.cuh"
 #include "kernels.h"
 #include "linear2d.cuh"
+#include "medium2d.cuh"
 #include "sharpclaw.cuh"
 
 namespace claw {
@@ -170,18 +171,20 @@ constexpr bool classic2d_fits(int bw) {
   return classic2d_smem<RP, R>(bw) + 1024 <= 48 * 1024;
 }
 
-// the classic step runs on the per-face path with a capacity, and in 2D for
-// solvers whose transverse split needs the neighbouring cells' media
+// the classic step runs on the per-face path with a capacity, except for 2D
+// acoustics in a varying medium, whose own kernel has it
+template <class RP, int ND>
+constexpr bool medium_kernel() { return ND == 2 && trans_aux_rp<RP>::value; }
 template <class RP, int ND>
 inline bool uses_faces(int capa) {
-  return ND <= 2 && (capa >= 0 || (ND == 2 && trans_aux_rp<RP>::value));
+  return ND <= 2 && capa >= 0 && !medium_kernel<RP, ND>();
 }
 
 template <class RP, typename R, int ND>
 struct Launchers {
   static cudaError_t classic(const LaunchArgs& a) {
     const MConsts<R>& C = *(const MConsts<R>*)a.consts;
-    if constexpr (ND <= 2) {
+    if constexpr (ND <= 2 && !medium_kernel<RP, ND>()) {
       if (uses_faces<RP, ND>(C.capa)) {
         const int nx = a.n3[0], ny = ND == 2 ? a.n3[1] : 1;
         const size_t fx = faces_sweep_threads(ND, nx, ny, 0), fy = faces_sweep_threads(ND, nx, ny, 1);
@@ -208,6 +211,14 @@ struct Launchers {
       else
         classic3d_kernel<RP, R, false><<<grid, 32 * kXSweepLines, 0, a.stream>>>(a.members, C, L);
       return cudaGetLastError();
+    } else if constexpr (medium_kernel<RP, ND>()) {
+      const bool fast = C.lim == CLAW_LIM_MC && C.order == 2 && C.transverse == 2 && a.sweep == 0;
+      if (a.bw != 64 && a.bw != 128) return cudaErrorInvalidValue;
+      if (a.bw == 128)
+        return fast ? reg2d(medium2d_kernel<RP, R, 128, true>, a, C)
+                    : reg2d(medium2d_kernel<RP, R, 128, false>, a, C);
+      return fast ? reg2d(medium2d_kernel<RP, R, 64, true>, a, C)
+                  : reg2d(medium2d_kernel<RP, R, 64, false>, a, C);
     } else if constexpr (ND == 2 && RP::MA > 0) {
       // 2D solvers with aux fields have normal solves only (SharpClaw)
       (void)C;
@@ -225,6 +236,13 @@ struct Launchers {
         return classic2d<true>(a, C);
       return classic2d<false>(a, C);
     }
+    return cudaGetLastError();
+  }
+  // one launch of a register-resident 2D kernel (a block per tile)
+  template <class K>
+  static cudaError_t reg2d(K kern, const LaunchArgs& a, const MConsts<R>& C) {
+    const int threads = 32 * reg_tile(sizeof(R) == 8 ? 0 : 1, a.bw).warps;
+    kern<<<launch_grid(a.ntiles_total), threads, 0, a.stream>>>(a.members, a.tiles, C, a.h, a.sweep);
     return cudaGetLastError();
   }
   // FAST (FP32 only): the common settings fixed at compile time
@@ -273,14 +291,9 @@ struct Launchers {
   static cudaError_t classic2d(const LaunchArgs& a, const MConsts<R>& C) {
     if constexpr (ND == 2 && is_linear_rp<RP, R>::value) {
       // bits do not depend on FAST or on the width (explicit rounding)
-      const unsigned grid = (unsigned)launch_grid(a.ntiles_total);
-      if (a.bw == 128)
-        linear2d_kernel<RP, R, 128, FAST><<<grid, 32, 0, a.stream>>>(a.members, a.tiles, C, a.h, a.sweep);
-      else if (a.bw == 64)
-        linear2d_kernel<RP, R, 64, FAST><<<grid, 32, 0, a.stream>>>(a.members, a.tiles, C, a.h, a.sweep);
-      else
-        return cudaErrorInvalidValue;
-      return cudaGetLastError();
+      if (a.bw == 128) return reg2d(linear2d_kernel<RP, R, 128, FAST>, a, C);
+      if (a.bw == 64) return reg2d(linear2d_kernel<RP, R, 64, FAST>, a, C);
+      return cudaErrorInvalidValue;
     } else if constexpr (ND == 2 && RP::MA == 0 && (!FAST || (sizeof(R) == 4 && RP::M <= 3))) {
       if constexpr (classic2d_fits<RP, R>(128)) {
         if (a.bw == 128) {
@@ -413,6 +426,10 @@ KernelSet make_set(bool has_char) {
   k.source = &Launchers<RP, R, ND>::source;
   k.blocks3 = &Launchers<RP, R, ND>::blocks3;
   k.max_bw = classic2d_fits<RP, R>(128) ? 128 : 64;
+  k.reg_kernel = ND == 2 && (is_linear_rp<RP, R>::value || medium_kernel<RP, ND>());
+  constexpr int prec = sizeof(R) == 8 ? 0 : 1;
+  k.tx64 = k.reg_kernel ? reg_tile(prec, 64).tx : 64 - 4;
+  k.tx128 = k.reg_kernel ? reg_tile(prec, 128).tx : 128 - 4;
   constexpr size_t lim = kSmemPerBlock;
   k.sharp_shapes = (sharp_smem_bytes<RP, R, 2, 16, 8, 3>() <= lim ? 1 : 0) |
                    (sharp_smem_bytes<RP, R, 2, 32, 4, 3>() <= lim ? 2 : 0) |

@@ -2,20 +2,21 @@
 // systems (advection, acoustics) in strength form (linear.cuh), one launch per
 // attempt (two for a dimensionally split step).
 //
-// A warp owns a strip of BW - 4 columns (BW / 32 columns per lane, two halo
-// columns on each side) and walks a chunk of rows: x neighbours are the
+// A warp owns a strip of columns (one, two or four per lane, two halo columns
+// on each side; reg_tile) and walks a chunk of rows: x neighbours are the
 // lane's own columns or come by warp shuffles, y neighbours are the lane's
 // values of earlier rows, so there is no shared-memory exchange and no
-// barrier.  With row R loaded the warp has tau_x of row R, tau_y of row R - 2
+// barrier in the walk.  With row R loaded the warp has tau_x of row R, tau_y of row R - 2
 // and finishes row R - 2.  Products and sums are written as explicit fused
 // multiply-adds, so every strip width and chunk height gives the same bits.
 //
-// What bounds it: FP64 the FP64 pipe (67 % on average at 1000 x 750, one wave
-// of 595 warps; about 45 FP64 instructions per column and row against some 250
-// of the vector form); FP32 issue and latency (53 % issue at 4096 x 3072,
-// 154 registers).  Acoustics 1000 x 750 FP64 368 -> 124 us/step, 4095 x 4000
-// FP32 373 -> 155 us, 1024^2 FP32 38.6 -> 32.3 us against the shared-memory
-// row walk of classic2d_kernel.
+// What bounds it: FP64 the FP64 pipe (67 % on average at 1000 x 750 in one
+// wave of two-column warps; about 45 FP64 instructions per column and row
+// against some 250 of the vector form); FP32 issue and latency (53 % issue at
+// 4096 x 3072, 154 registers), small grids the latency of an attempt.
+// Acoustics 1000 x 750 FP64 368 -> 115 us/step, 64^2 FP64 63 -> 28 us, 4095 x
+// 4000 FP32 373 -> 155 us, 1024^2 FP32 38.6 -> 31.6 us against the
+// shared-memory row walk of classic2d_kernel.
 #pragma once
 
 #include "kernels.h"
@@ -39,15 +40,36 @@ __device__ __forceinline__ void st2(double* p, double a, double b) {
   *(double2*)p = make_double2(a, b);
 }
 
+// one column or a pair of a row
+template <int N, typename R>
+__device__ __forceinline__ void ld_pair(const R* p, bool vec, R& a, R& b) {
+  if (N > 1 && vec) {
+    ld2(p, a, b);
+  } else {
+    a = __ldg(p);
+    if (N > 1) b = __ldg(p + 1);
+  }
+}
+template <typename R>
+__device__ __forceinline__ void st_pair(R* p, bool two, bool vec, R a, R b) {
+  if (two && vec) {
+    st2(p, a, b);
+  } else {
+    p[0] = a;
+    if (two) p[1] = b;
+  }
+}
+
 // sweep: 0 the unsplit step (slot 0 -> 1); dimensional splitting: 1 the x
 // sweeps (slot 0 -> 1), 2 the y sweeps (slot 1 -> 2).  FAST: the MC limiter,
 // second order and transverse mode 2 fixed at compile time.
 template <class RP, typename R, int BW, bool FAST>
-__global__ void __launch_bounds__(32)
+__global__ void __launch_bounds__(32 * reg_tile(sizeof(R) == 8 ? 0 : 1, BW).warps)
     linear2d_kernel(const Member* __restrict__ members, const Tile* __restrict__ tiles,
                     const MConsts<R> C, int H, int sweep) {
   using LS = Lin<RP, R>;
-  constexpr int M = RP::M, NS = LS::NS, N = BW / 32;
+  constexpr RegTile RT = reg_tile(sizeof(R) == 8 ? 0 : 1, BW);
+  constexpr int M = RP::M, NS = LS::NS, N = RT.n, WL = 32 * N;  // columns per lane, per warp
   constexpr bool VEL = LS::VEL;
   constexpr int U = VEL ? 1 : 0, V = VEL ? 2 : 0;
   constexpr unsigned FULL = 0xffffffffu;
@@ -56,18 +78,18 @@ __global__ void __launch_bounds__(32)
   const Member& mb = members[tl.member];
   DevCtl* ctl = mb.ctl;
   if (ctl->done) return;  // the whole block
-  const int lane = threadIdx.x;
-  if (lane < 2) {
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x < 2) {
     LS::consts(C, lane, ctl->dt / ctl->dx[lane], K[lane]);
     T[lane] = K[lane];  // transverse terms act on -tau/2
     T[lane].t0 *= R(-0.5);
     T[lane].t1 *= R(-0.5);
   }
-  __syncwarp();
+  __syncthreads();
   const int cur = ctl->cur, nbuf = ctl->nbuf;
   const int nx = mb.nx, ny = mb.ny;
-  const Classic2dLayout L = classic2d_layout(nx, ny, BW, H);
-  const int c0 = (tl.tile % L.nsx) * L.TX, ch = tl.tile / L.nsx;
+  const Classic2dLayout L = classic2d_layout(nx, ny, RT.tx, H);
+  const int c0 = (tl.tile % L.nsx) * L.TX + (threadIdx.x >> 5) * (WL - 4), ch = tl.tile / L.nsx;
   const int r0 = (int)(((long long)ch * ny) / L.nch);
   const int r1 = (int)(((long long)(ch + 1) * ny) / L.nch);
   const bool dox = sweep != 2, doy = sweep != 1;
@@ -88,14 +110,8 @@ __global__ void __launch_bounds__(32)
 #pragma unroll
       for (int k = 0; k < M; ++k) {
 #pragma unroll
-        for (int c = 0; c < N; c += 2) {
-          if (vec) {
-            ld2(p + k * plane + c, v[c][k], v[c + 1][k]);
-          } else {
-            v[c][k] = __ldg(p + k * plane + c);
-            v[c + 1][k] = __ldg(p + k * plane + c + 1);
-          }
-        }
+        for (int c = 0; c < N; c += 2)
+          ld_pair<N>(p + k * plane + c, vec, v[c][k], v[c + (N > 1)][k]);
       }
     } else {
 #pragma unroll
@@ -119,8 +135,9 @@ __global__ void __launch_bounds__(32)
   }
   int bad = 0;
   R qn[N][M];
-  load(r0 - 2, qn);
-  for (int r = r0 - 2; r <= r1 + 1; ++r) {
+  if (c0 < nx) load(r0 - 2, qn);
+  // (a warp whose strip starts past the grid has nothing to do)
+  for (int r = c0 < nx ? r0 - 2 : r1 + 2; r <= r1 + 1; ++r) {
     R acc0[N][M], tx[N], ty[N], zo[N];
 #pragma unroll
     for (int c = 0; c < N; ++c) {
@@ -203,19 +220,14 @@ __global__ void __launch_bounds__(32)
 #pragma unroll
       for (int c = 0; c < N; c += 2) {
         const int l = N * lane + c;
-        if (l >= 2 && l < BW - 2 && g0 + c < nx) {
-          const bool two = g0 + c + 1 < nx;
+        if (l >= 2 && l < WL - 2 && g0 + c < nx) {
+          const bool two = N > 1 && g0 + c + 1 < nx;
 #pragma unroll
           for (int k = 0; k < M; ++k) {
-            R* o = qo + k * plane + (size_t)(r - 2) * nx + (g0 + c);
-            bad |= not_finite(acc2[c][k]);
-            if (two) bad |= not_finite(acc2[c + 1][k]);
-            if (two && vec) {
-              st2(o, acc2[c][k], acc2[c + 1][k]);
-            } else {
-              o[0] = acc2[c][k];
-              if (two) o[1] = acc2[c + 1][k];
-            }
+            const R a = acc2[c][k], b = acc2[c + (N > 1)][k];
+            bad |= not_finite(a);
+            if (two) bad |= not_finite(b);
+            st_pair(qo + k * plane + (size_t)(r - 2) * nx + (g0 + c), two, vec, a, b);
           }
         }
       }

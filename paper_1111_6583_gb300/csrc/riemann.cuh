@@ -956,7 +956,8 @@ struct RpElasticity {
 // impedance and speed, the right-going one the right cell's; the transverse
 // split of a fluctuation held by a cell solves the transverse Riemann
 // problems with its neighbours below and above (TRANS_AUX: it needs their
-// media, so 2D classic steps with this solver run the per-face path).
+// media, so 2D classic steps with this solver have a kernel of their own,
+// medium2d.cuh).
 // ---------------------------------------------------------------------------
 template <typename R, int ND>
 struct RpAcousticsVC {
@@ -1008,27 +1009,6 @@ struct RpAcousticsVC {
                                                const R (&)[M], R (&bm)[M], R (&bp)[M]) {
 #pragma unroll
     for (int k = 0; k < M; ++k) bm[k] = bp[k] = R(0);
-  }
-  // B^- a: down-going wave between the cell below (am_) and the cell (ac);
-  // B^+ a: up-going wave between the cell and the one above (ap_)
-  template <int DIR>
-  __device__ static __forceinline__ void trans_aux(const MConsts<R>&, const R* am_, const R* ac,
-                                                   const R* ap_, const R (&a)[M], R (&bm)[M],
-                                                   R (&bp)[M]) {
-    constexpr int t = Dirs<ND, DIR>::t < 0 ? 0 : Dirs<ND, DIR>::t;
-    const R Zm = am_[0] * am_[1], Zc = ac[0] * ac[1], Zp = ap_[0] * ap_[1];
-#pragma unroll
-    for (int k = 0; k < M; ++k) bm[k] = bp[k] = R(0);
-    // one reciprocal for both impedance sums (positive, of the media's scale,
-    // so their product stays in range)
-    const R sm = Zm + Zc, sp = Zc + Zp;
-    const R inv = FM<R>::rcp(sm * sp);
-    const R b1 = (-a[0] + Zc * a[t]) * (sp * inv);
-    const R b2 = (a[0] + Zc * a[t]) * (sm * inv);
-    bm[0] = am_[1] * b1 * Zm;
-    bm[t] = -am_[1] * b1;
-    bp[0] = ap_[1] * b2 * Zp;
-    bp[t] = ap_[1] * b2;
   }
   template <int DIR>
   __device__ static __forceinline__ void char_ctx(const MConsts<R>&, const R (&)[M],
