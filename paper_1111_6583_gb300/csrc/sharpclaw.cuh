@@ -18,74 +18,103 @@
 #include "async_copy.cuh"
 #include "kernels.h"
 #include "riemann.cuh"
+#include "vec.cuh"
 #include "weno_hi.cuh"
 
 namespace claw {
 
-// Both Jiang-Shu WENO5 values at the interface between cells c and d of the
-// six cell averages a..f: the left-biased one at the right edge of c (um)
-// and the right-biased one at the left edge of d (up), as numerator and
-// denominator.  The two use the same candidates from stencils (b, c, d) and
-// (c, d, e) and the same second differences of those stencils, computed
-// once here; candidates are kept times 6 (the 6 moves to the denominator).
-template <typename R>
-__device__ __forceinline__ void weno5_pair(R a, R b, R c, R d, R e, R f, R eps, R& nm, R& dm,
-                                           R& np, R& dp) {
-  const R p0 = R(2) * a - R(7) * b + R(11) * c;   // (a, b, c) at the right edge of c
-  const R p1 = R(2) * d + R(5) * c - b;           // (b, c, d) at the c|d edge
-  const R p2 = R(2) * c + R(5) * d - e;           // (c, d, e) at the c|d edge
-  const R p3 = R(2) * f - R(7) * e + R(11) * d;   // (d, e, f) at the left edge of d
-  const R k13 = R(13) / R(12);
-  const R t0 = a - R(2) * b + c, t1 = b - R(2) * c + d, t2 = c - R(2) * d + e,
-          t3 = d - R(2) * e + f;
-  const R h0 = k13 * (t0 * t0), h1 = k13 * (t1 * t1), h2 = k13 * (t2 * t2),
-          h3 = k13 * (t3 * t3);
-  const R u0 = a - R(4) * b + R(3) * c, u1 = b - d, u2 = R(3) * c - R(4) * d + e;
-  const R v0 = f - R(4) * e + R(3) * d, v1 = e - c, v2 = R(3) * d - R(4) * c + b;
-  const R e0 = eps + (h0 + R(0.25) * (u0 * u0)), e1 = eps + (h1 + R(0.25) * (u1 * u1)),
-          e2 = eps + (h2 + R(0.25) * (u2 * u2));
-  const R g0 = eps + (h3 + R(0.25) * (v0 * v0)), g1 = eps + (h2 + R(0.25) * (v1 * v1)),
-          g2 = eps + (h1 + R(0.25) * (v2 * v2));
-  // alpha_k = d_k / beta_k^2 multiplied through by the product of the three
-  const R s0 = e0 * e0, s1 = e1 * e1, s2 = e2 * e2;
-  const R w0 = R(0.1) * (s1 * s2), w1 = R(0.6) * (s0 * s2), w2 = R(0.3) * (s0 * s1);
-  nm = w0 * p0 + w1 * p1 + w2 * p2;
-  dm = R(6) * (w0 + w1 + w2);
-  const R z0 = g0 * g0, z1 = g1 * g1, z2 = g2 * g2;
-  const R y0 = R(0.1) * (z1 * z2), y1 = R(0.6) * (z0 * z2), y2 = R(0.3) * (z0 * z1);
-  np = y0 * p3 + y1 * p2 + y2 * p1;
-  dp = R(6) * (y0 + y1 + y2);
+// Both Jiang-Shu WENO5 values at the interface between cells c and d of six
+// cell averages a .. f, from their five first differences D: the left-biased
+// value at the right edge of c is c + nl / dl, the right-biased one at the
+// left edge of d is d - nr / dr.  The two share the candidates and second
+// differences of the stencils (b, c, d) and (c, d, e).  Differences in place
+// of averages take fewer operations (58 against 86 per pair) and cancel once,
+// before the products.  Smoothness indicators are kept times 4 (eps4 = 4 eps)
+// and candidates times 6 (the 6 moves to the denominator).
+template <typename V, typename R>
+__device__ __forceinline__ void weno5_diff(const V (&D)[5], R eps4, V& nl, V& dl, V& nr, V& dr) {
+  const V two = V(R(2)), mtwo = V(R(-2)), k13 = V(R(13) / R(3)), e4 = V(eps4);
+  const V t0 = vsub(D[1], D[0]), t1 = vsub(D[2], D[1]), t2 = vsub(D[3], D[2]),
+          t3 = vsub(D[4], D[3]);
+  const V h0 = vfma(vmul(k13, t0), t0, e4), h1 = vfma(vmul(k13, t1), t1, e4),
+          h2 = vfma(vmul(k13, t2), t2, e4), h3 = vfma(vmul(k13, t3), t3, e4);
+  const V u0 = vfma(two, D[1], t0), u1 = vadd(D[1], D[2]), u2 = vfma(mtwo, D[2], t2);
+  const V v0 = vfma(mtwo, D[3], t3), v1 = vadd(D[2], D[3]), v2 = vfma(two, D[2], t1);
+  const V e0 = vfma(u0, u0, h0), e1 = vfma(u1, u1, h1), e2 = vfma(u2, u2, h2);
+  const V g0 = vfma(v0, v0, h3), g1 = vfma(v1, v1, h2), g2 = vfma(v2, v2, h1);
+  // weights d_k / beta_k^2 (1/10, 6/10, 3/10) times the product of the three
+  auto side = [&](V e0, V e1, V e2, V p0, V p1, V p2, V& n, V& d) {
+    const V s1 = vmul(e1, e1), s2 = vmul(e2, e2), a = vmul(vmul(V(R(3)), e0), e0);
+    const V s12 = vmul(s1, s2), b = vadd(s2, s2);
+    n = vfma(a, vfma(b, p1, vmul(s1, p2)), vmul(s12, p0));
+    d = vmul(V(R(6)), vfma(a, vadd(b, s1), s12));
+  };
+  const V five = V(R(5)), four = V(R(4)), mone = V(R(-1));
+  side(e0, e1, e2, vfma(five, D[1], vmul(mtwo, D[0])), vfma(two, D[2], D[1]),
+       vfma(four, D[2], vmul(mone, D[3])), nl, dl);
+  side(g0, g1, g2, vfma(five, D[3], vmul(mtwo, D[4])), vfma(two, D[2], D[3]),
+       vfma(four, D[2], vmul(mone, D[1])), nr, dr);
 }
 
-// n / d for N pairs.  In FP64 with one division: 1/d_i = (prod_{j<i} d_j)
-// (prod_{j>i} d_j) / prod_j d_j, taken only when every partial product is a
-// positive normal number (no overflow, underflow or lost precision), else N
-// divisions.
+// n / d for N pairs.  FP64: the reciprocals from the hardware seed and one
+// step of Halley's iteration (x y = 1 - e: y (1 + e + e^2), error e^3 of a
+// seed good to 20 bits, so correct to about one rounding: three FP64
+// instructions against about eight of a division), taken only when every
+// divisor is well inside the normal range, else N divisions.
 template <typename R, int N>
 __device__ __forceinline__ void div_many(const R (&n)[N], const R (&d)[N], R (&q)[N]) {
-  if constexpr (sizeof(R) == 8 && N > 1) {
-    R pre[N];
-    R prod = d[0];
-    bool normal = pos_normal(prod);
-    pre[0] = R(1);
+  if constexpr (sizeof(R) == 8) {
+    bool normal = true;
 #pragma unroll
-    for (int i = 1; i < N; ++i) {
-      pre[i] = prod;
-      prod = prod * d[i];
-      normal = normal && pos_normal(prod);
-    }
+    for (int i = 0; i < N; ++i)
+      normal = normal && (unsigned)(__double2hiint(d[i]) - 0x10000000) < 0x60000000u;
     if (normal) {
-      R suf = FM<R>::rcp(prod);
 #pragma unroll
-      for (int i = N - 1; i >= 0; --i) {
-        q[i] = n[i] * (i == 0 ? suf : suf * pre[i]);
-        suf = suf * d[i];
+      for (int i = 0; i < N; ++i) {
+        double y;
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d[i]));
+        const double e = fma(-d[i], y, 1.0);
+        q[i] = n[i] * fma(y, fma(e, e, e), y);
       }
       return;
     }
   }
 #pragma unroll
   for (int i = 0; i < N; ++i) q[i] = FM<R>::div(n[i], d[i]);
+}
+
+// the WENO5 pairs of M fields from their differences w[field][5]: corrections
+// to the average of the cell on each side (um: add to c, up: subtract from d)
+template <typename R, int M>
+__device__ __forceinline__ void weno5_fields(const R (&w)[M][5], R eps, R (&um)[M], R (&up)[M]) {
+  R nn[2 * M], dd[2 * M], vv[2 * M];
+  const R eps4 = R(4) * eps;
+  if constexpr (sizeof(R) == 4) {
+    // two fields per packed instruction (an odd last field alone)
+#pragma unroll
+    for (int k = 0; k + 1 < M; k += 2) {
+      F2 D[5], a, b, c, d;
+#pragma unroll
+      for (int j = 0; j < 5; ++j) D[j] = F2(w[k][j], w[k + 1][j]);
+      weno5_diff<F2, float>(D, eps4, a, b, c, d);
+      a.get(nn[k], nn[k + 1]);
+      b.get(dd[k], dd[k + 1]);
+      c.get(nn[M + k], nn[M + k + 1]);
+      d.get(dd[M + k], dd[M + k + 1]);
+    }
+    if constexpr (M % 2 == 1)
+      weno5_diff<R, R>(w[M - 1], eps4, nn[M - 1], dd[M - 1], nn[2 * M - 1], dd[2 * M - 1]);
+  } else {
+#pragma unroll
+    for (int k = 0; k < M; ++k)
+      weno5_diff<R, R>(w[k], eps4, nn[k], dd[k], nn[M + k], dd[M + k]);
+  }
+  div_many<R, 2 * M>(nn, dd, vv);
+#pragma unroll
+  for (int k = 0; k < M; ++k) {
+    um[k] = vv[k];
+    up[k] = vv[M + k];
+  }
 }
 
 // WENO of order 2 RW - 1 (7 .. 17; WENO5 takes weno5_pair): left-biased value at the right edge of cell
@@ -105,6 +134,24 @@ __device__ __forceinline__ R weno_edge(const R (&w)[NV], R eps) {
   else return weno17<R>(v, eps);
 }
 
+// Resident blocks the registers are held to (0: the compiler's choice).  The
+// FP32 WENO5 stage waits on its tile loads and barriers, and more warps pay
+// for the few spills: with four 256-thread blocks per SM (64 registers)
+// 1500 x 700 shock-bubble 270 us/step, three or five 295, left to the compiler
+// (80 registers) 310; six 128-thread blocks (80 registers) suit small grids.
+template <typename R, int TX, int TY, int RW>
+__host__ __device__ constexpr int sharp_minb() {
+  return sizeof(R) == 4 && RW == 3 && TY > 1 ? (TX * TY == 256 ? 4 : 6) : 0;
+}
+// Values of the interfaces' Roe averages kept per cell.  FP64: they save some
+// 30 of 560 FP64 instructions per interface; FP32: forming them at each
+// interface is cheaper than another barrier and its shared memory (270 against
+// 280 us/step).
+template <class RP, typename R, int RW>
+__host__ __device__ constexpr int sharp_ncp() {
+  return RW == 3 && sizeof(R) == 8 ? char_prep_n<RP>() : 0;
+}
+
 // static shared memory of sharp_stage_kernel (the arrays declared in it)
 template <class RP, typename R, int ND, int TX, int TY, int RW>
 constexpr size_t sharp_smem_bytes() {
@@ -116,13 +163,15 @@ constexpr size_t sharp_smem_bytes() {
   constexpr int HXP0 = (OX + HX + A - 1) / A * A;
   constexpr int HXP = !kStageRows ? HX : ((HXP0 / A) % 2 == 1 ? HXP0 : HXP0 + A);
   constexpr int NE = (ND == 2) ? (TX + 1) * TY + TX * (TY + 1) : TX + 1;
+  constexpr int NCP = sharp_ncp<RP, R, RW>();
   return sizeof(R) * ((size_t)M * HY * HXP + (size_t)MAS * (MA > 0 ? HY * HXP : 1) +
-                      (size_t)HY * HX + 4 * (size_t)M * NE + 3) +
+                      (size_t)HY * HX + (size_t)(NCP > 0 ? NCP * HY * HX : 1) +
+                      4 * (size_t)M * NE + 3) +
          3 * sizeof(int) + 8;
 }
 
 template <class RP, typename R, int ND, int TX, int TY, int RW>
-__global__ void __launch_bounds__(TX * TY)
+__global__ void __launch_bounds__(TX * TY, sharp_minb<R, TX, TY, RW>())
     sharp_stage_kernel(const Member* __restrict__ members, const Tile* __restrict__ tiles,
                        int ntiles_total, const MConsts<R> C, const StageOp op) {
   constexpr int M = RP::M, MW = RP::MW, MA = RP::MA, NC = RP::NCTX;
@@ -145,7 +194,7 @@ __global__ void __launch_bounds__(TX * TY)
   // step); rows padded to an odd number of 16-byte units, so that a column
   // of cells spreads over the shared-memory banks (the y-interface phase
   // reads down columns).  Without staging the rows are HX values, OX = 0.
-  constexpr bool kStageRows = NT <= 128;
+  constexpr bool kStageRows = TX * TY <= 128;
   constexpr int A = 16 / (int)sizeof(R), OX = kStageRows ? (A - G % A) % A : 0;
   constexpr int HXP0 = (OX + HX + A - 1) / A * A;
   constexpr int HXP = !kStageRows ? HX : ((HXP0 / A) % 2 == 1 ? HXP0 : HXP0 + A);
@@ -154,6 +203,9 @@ __global__ void __launch_bounds__(TX * TY)
   __shared__ __align__(16) R At[MAS][MA > 0 ? HY : 1][MA > 0 ? HXP : 1];
   __shared__ __align__(8) unsigned long long s_bar;  // completes the staging copies
   __shared__ R Kt[HY][HX];  // capacity kappa (when the method has one)
+  // per-cell part of the interfaces' Roe averages (WENO5, characteristic form)
+  constexpr int NCP = sharp_ncp<RP, R, RW>(), NCPS = NCP > 0 ? NCP : 1;
+  __shared__ R Pc[NCPS][NCP > 0 ? HY : 1][NCP > 0 ? HX : 1];
   __shared__ R EL[M][NE];  // left edge value of the cell right of an interface
   __shared__ R ER[M][NE];  // right edge value of the cell left of an interface
   __shared__ R FM[M][NE];  // A^- dQ at the interface
@@ -178,8 +230,8 @@ __global__ void __launch_bounds__(TX * TY)
     if (tid == 0) {
       s_done = ctl->done;
       s_dt = (R)ctl->dt;
-      s_idn[0] = (R)(1.0 / ctl->dx[0]);
-      s_idn[1] = (R)(1.0 / ctl->dx[1]);
+      s_idn[0] = (R)ctl->idx[0];  // 1/dx, divided once on the host
+      s_idn[1] = (R)ctl->idx[1];
       s_cur = ctl->cur;
       s_nbuf = ctl->nbuf;
     }
@@ -267,6 +319,24 @@ __global__ void __launch_bounds__(TX * TY)
       __syncthreads();
     }
     const bool skip = bad != 0;
+    if constexpr (NCP > 0) {
+      if (C.char_decomp) {
+        // the cells beside an interface: one more than the tile on each side
+        constexpr int WX = TX + 2, WY = (ND == 2) ? TY + 2 : 1;
+        for (int idx = tid; idx < WX * WY; idx += NT) {
+          const int hi = G - 1 + idx % WX, hj = (ND == 2) ? G - 1 + idx / WX : 0;
+          const bool xin = hi >= G && hi < G + TX, yin = ND == 1 || (hj >= G && hj < G + TY);
+          if (!xin && !yin) continue;  // corners (not loaded cell by cell)
+          R v[M], p[NCPS];
+#pragma unroll
+          for (int k = 0; k < M; ++k) v[k] = Qt[k][hj][OX + hi];
+          RP::char_prep(C, v, p);
+#pragma unroll
+          for (int k = 0; k < NCP; ++k) Pc[k][hj][hi] = p[k];
+        }
+        __syncthreads();
+      }
+    }
 
     R L[M];
 #pragma unroll
@@ -290,49 +360,69 @@ __global__ void __launch_bounds__(TX * TY)
         for (int k = 0; k < M; ++k) cell[k6][k] = Qt[k][hj][OX + hi];
       }
       R wm[M], wp[M];
-      if (C.char_decomp) {
+      if constexpr (RW == 3) {
+        // WENO5 on the differences of the six cells (of their characteristic
+        // components: the projection is linear); corrections to the two cells
+        R df[5][M], w[M][5], um[M], up[M];
+#pragma unroll
+        for (int k6 = 0; k6 < 5; ++k6)
+#pragma unroll
+          for (int k = 0; k < M; ++k) df[k6][k] = cell[k6 + 1][k] - cell[k6][k];
+        if (C.char_decomp) {
+          R x[NC];
+          if constexpr (NCP > 0) {
+            const int hil = (dir == 0) ? G + a - 1 : G + b, hir = (dir == 0) ? G + a : G + b;
+            const int hjl = (dir == 0) ? ((ND == 2) ? G + b : 0) : G + a - 1;
+            const int hjr = (dir == 0) ? ((ND == 2) ? G + b : 0) : G + a;
+            R pl[NCPS], pr[NCPS];
+#pragma unroll
+            for (int k = 0; k < NCP; ++k) {
+              pl[k] = Pc[k][hjl][hil];
+              pr[k] = Pc[k][hjr][hir];
+            }
+            RP::template char_ctx_pc<dir>(C, cell[RW - 1], cell[RW], pl, pr, x);
+          } else {
+            RP::template char_ctx<dir>(C, cell[RW - 1], cell[RW], x);
+          }
+#pragma unroll
+          for (int k6 = 0; k6 < 5; ++k6) {
+            R v[M];
+            RP::template to_char<dir>(C, x, df[k6], v);
+#pragma unroll
+            for (int k = 0; k < M; ++k) w[k][k6] = v[k];
+          }
+          weno5_fields<R, M>(w, C.weno_eps, um, up);
+          RP::template from_char<dir>(C, x, um, wm);
+          RP::template from_char<dir>(C, x, up, wp);
+        } else {
+#pragma unroll
+          for (int k = 0; k < M; ++k)
+#pragma unroll
+            for (int k6 = 0; k6 < 5; ++k6) w[k][k6] = df[k6][k];
+          weno5_fields<R, M>(w, C.weno_eps, wm, wp);
+        }
+#pragma unroll
+        for (int k = 0; k < M; ++k) {
+          wm[k] = cell[RW - 1][k] + wm[k];
+          wp[k] = cell[RW][k] - wp[k];
+        }
+      } else if (C.char_decomp) {
         R x[NC];
         R w[NS][M];
         RP::template char_ctx<dir>(C, cell[RW - 1], cell[RW], x);
 #pragma unroll
         for (int k6 = 0; k6 < NS; ++k6) RP::template to_char<dir>(C, x, cell[k6], w[k6]);
         R um[M], up[M];
-        if constexpr (RW == 3) {
-          R nn[2 * M], dd[2 * M], vv[2 * M];
 #pragma unroll
-          for (int k = 0; k < M; ++k)
-            weno5_pair<R>(w[0][k], w[1][k], w[2][k], w[3][k], w[4][k], w[5][k], C.weno_eps,
-                          nn[k], dd[k], nn[M + k], dd[M + k]);
-          div_many<R, 2 * M>(nn, dd, vv);
+        for (int k = 0; k < M; ++k) {
+          R line[NS];
 #pragma unroll
-          for (int k = 0; k < M; ++k) {
-            um[k] = vv[k];
-            up[k] = vv[M + k];
-          }
-        } else {
-#pragma unroll
-          for (int k = 0; k < M; ++k) {
-            R line[NS];
-#pragma unroll
-            for (int k6 = 0; k6 < NS; ++k6) line[k6] = w[k6][k];
-            um[k] = weno_edge<RW, false>(line, C.weno_eps);
-            up[k] = weno_edge<RW, true>(line, C.weno_eps);
-          }
+          for (int k6 = 0; k6 < NS; ++k6) line[k6] = w[k6][k];
+          um[k] = weno_edge<RW, false>(line, C.weno_eps);
+          up[k] = weno_edge<RW, true>(line, C.weno_eps);
         }
         RP::template from_char<dir>(C, x, um, wm);
         RP::template from_char<dir>(C, x, up, wp);
-      } else if constexpr (RW == 3) {
-        R nn[2 * M], dd[2 * M], vv[2 * M];
-#pragma unroll
-        for (int k = 0; k < M; ++k)
-          weno5_pair<R>(cell[0][k], cell[1][k], cell[2][k], cell[3][k], cell[4][k], cell[5][k],
-                        C.weno_eps, nn[k], dd[k], nn[M + k], dd[M + k]);
-        div_many<R, 2 * M>(nn, dd, vv);
-#pragma unroll
-        for (int k = 0; k < M; ++k) {
-          wm[k] = vv[k];
-          wp[k] = vv[M + k];
-        }
       } else {
 #pragma unroll
         for (int k = 0; k < M; ++k) {
