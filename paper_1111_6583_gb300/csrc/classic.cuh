@@ -373,10 +373,7 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 && RP::M <= 2) ? (K >= 8 ?
     const int t0 = tl.tile * T;
     if (t0 + sub0 * WC >= nx) continue;
     const int cur = ctl->cur, nbuf = ctl->nbuf;
-    // FP32: one multiply by the stored 1/dx; FP64: the exact quotient
-    R dtdx;
-    if constexpr (sizeof(R) == 4) dtdx = (R)(ctl->dt * ctl->idx[0]);
-    else dtdx = ctl->dt / ctl->dx[0];
+    const R dtdx = dt_over_dx<R>(ctl, 0);
     const R* __restrict__ q = (const R*)mb.q[cur];
     R* __restrict__ qo = (R*)mb.q[(cur + 1) % nbuf];
     const R* __restrict__ aux = (const R*)mb.aux;
@@ -684,10 +681,9 @@ __global__ void __launch_bounds__(BW)
     DevCtl* ctl = mb.ctl;
     if (l == 0) {
       s_done = ctl->done;
-      const double dtd = ctl->dt;
-      s_k[0] = (R)(dtd / ctl->dx[0]);
-      s_k[1] = (R)(dtd / ctl->dx[1]);
-      s_k[2] = (R)(0.5 * (dtd / ctl->dx[0]) * (dtd / ctl->dx[1]));
+      s_k[0] = dt_over_dx<R>(ctl, 0);
+      s_k[1] = dt_over_dx<R>(ctl, 1);
+      s_k[2] = R(0.5) * s_k[0] * s_k[1];
       s_cur = ctl->cur;
       s_nbuf = ctl->nbuf;
     }

@@ -57,10 +57,48 @@ __device__ __forceinline__ double mc_half(double u, double a) {
   if ((ah ^ uh) < 0) m = 0ULL;
   return __longlong_as_double((long long)(m | ((unsigned long long)(unsigned)(ah & 0x80000000) << 32)));
 }
+// phi(u/a) a of the other limiters.  FP64: minima, maxima and doublings on
+// the bit patterns (of minmod and superbee nothing runs on the FP64 pipe); van
+// Leer's 2 u a / (u + a) by one Halley step from the hardware reciprocal where
+// the sum is well inside the normal range, else by division
+__device__ __forceinline__ float limit_general(int lim, float u, float a) {
+  return limited_strength<float>(lim, u, a);
+}
+__device__ __forceinline__ double limit_general(int lim, double u, double a) {
+  if (lim == CLAW_LIM_NONE) return a;
+  using U = unsigned long long;
+  const U m = 0x7fffffffffffffffULL, am = (U)fbits(a) & m, um = (U)fbits(u) & m;
+  const U lo = am < um ? am : um, hi = am < um ? um : am;
+  U g;
+  if (lim == CLAW_LIM_MINMOD) {
+    g = lo;
+  } else if (lim == CLAW_LIM_SUPERBEE) {
+    // max(min(2|u|, |a|), min(|u|, 2|a|)) = min(2 lo, hi); a value below
+    // 2^-1022 doubles as a denormal (a shift)
+    const U two = lo >= 0x0010000000000000ULL ? lo + 0x0010000000000000ULL : lo << 1;
+    g = two < hi ? two : hi;
+  } else {
+    const double au = fabs(u), aa = fabs(a), s = au + aa;
+    double r = 0.0;
+    if (am == 0 || um == 0) {
+      // no correction (and no division where the flow is at rest)
+    } else if ((unsigned)(__double2hiint(s) - 0x10000000) < 0x60000000u) {
+      double y;
+      asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(s));
+      const double e = fma(-s, y, 1.0);
+      r = (2.0 * au) * (aa * fma(y, fma(e, e, e), y));
+    } else {
+      r = FM<double>::div(2.0 * au * aa, s);
+    }
+    g = (U)fbits(r) & m;
+  }
+  if ((__double2hiint(a) ^ __double2hiint(u)) < 0 || am == 0 || um == 0) g = 0ULL;
+  return __longlong_as_double((long long)(g | ((U)fbits(a) & ~m)));
+}
 template <bool FAST, typename R>
 __device__ __forceinline__ R lin_limit(int lim, R u, R a) {
   if (FAST || lim == CLAW_LIM_MC) return mc_half(u, a);
-  return limited_strength<R>(lim, u, a);
+  return limit_general(lim, u, a);
 }
 
 // Per-attempt constants of one direction (computed once per block)
@@ -102,17 +140,17 @@ template <typename R, int ND>
 struct Lin<RpAcoustics<R, ND>, R> {
   static constexpr int M = ND + 1, NS = 2;
   static constexpr bool VEL = true;  // the normal velocity takes part
-  __device__ static void consts(const MConsts<R>& C, int d, double dtdx, LinK<R>& k) {
-    const double c = (double)C.aco_c, Z = (double)C.aco_Z, nu = c * dtdx;
-    k.c = (R)(0.5 * nu);
+  __device__ static void consts(const MConsts<R>& C, int d, R dtdx, LinK<R>& k) {
+    const R nu = C.aco_c * dtdx;
+    k.c = R(0.5) * nu;
     k.cm = R(0);
-    const double cf = 0.5 * nu * 0.5 * (1.0 - nu);
-    k.cf = C.order == 2 ? (R)(C.lim == CLAW_LIM_MC ? 2.0 * cf : cf) : R(0);
-    k.t0 = (R)(0.5 * nu);
-    k.t1 = (R)(0.5 * nu / Z);
-    k.d1 = (R)(nu / 6.0 - 0.5);
-    k.d2 = (R)(-nu / 12.0);
-    k.iz = (R)(1.0 / Z);
+    const R cf = k.c * (R(0.5) * (R(1) - nu));
+    k.cf = C.order == 2 ? (C.lim == CLAW_LIM_MC ? R(2) * cf : cf) : R(0);
+    k.t0 = k.c;
+    k.t1 = nu * C.aco_h;
+    k.d1 = nu * (R(1) / R(6)) - R(0.5);
+    k.d2 = nu * (R(-1) / R(12));
+    k.iz = R(2) * C.aco_h;
   }
   __device__ static R speed(const MConsts<R>& C, int) { return (R)fabs(C.aco_c); }
   // strengths of the face between states (pl, ul) and (pr, ur)
@@ -168,12 +206,12 @@ template <typename R, int ND>
 struct Lin<RpAdvection<R, ND>, R> {
   static constexpr int M = 1, NS = 1;
   static constexpr bool VEL = false;
-  __device__ static void consts(const MConsts<R>& C, int d, double dtdx, LinK<R>& k) {
-    const double v = (double)C.p[d], a = fabs(v) * dtdx;
-    k.c = (R)(v > 0.0 ? a : 0.0);
-    k.cm = (R)(v < 0.0 ? -a : 0.0);
-    const double cf = 0.5 * a * (1.0 - a);
-    k.cf = C.order == 2 ? (R)(C.lim == CLAW_LIM_MC ? 2.0 * cf : cf) : R(0);
+  __device__ static void consts(const MConsts<R>& C, int d, R dtdx, LinK<R>& k) {
+    const R v = C.p[d], a = (R)fabs(v) * dtdx;
+    k.c = v > R(0) ? a : R(0);
+    k.cm = v < R(0) ? -a : R(0);
+    const R cf = R(0.5) * a * (R(1) - a);
+    k.cf = C.order == 2 ? (C.lim == CLAW_LIM_MC ? R(2) * cf : cf) : R(0);
     k.t0 = k.c;
     k.t1 = -k.cm;
     k.d1 = k.d2 = k.iz = R(0);

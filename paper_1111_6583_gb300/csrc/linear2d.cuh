@@ -14,9 +14,11 @@
 // wave of two-column warps; about 45 FP64 instructions per column and row
 // against some 250 of the vector form); FP32 issue and latency (53 % issue at
 // 4096 x 3072, 154 registers), small grids the latency of an attempt.
-// Acoustics 1000 x 750 FP64 368 -> 115 us/step, 64^2 FP64 63 -> 28 us, 4095 x
-// 4000 FP32 373 -> 155 us, 1024^2 FP32 38.6 -> 31.6 us against the
-// shared-memory row walk of classic2d_kernel.
+// Acoustics 1000 x 750 FP64 368 -> 122 us/step, 64^2 FP64 63 -> 28 us, 700 x
+// 650 FP64 superbee 231 -> 83 us, 1024^2 FP32 38.6 -> 26.2 us against the
+// shared-memory row walk of classic2d_kernel.  Rows collect increments and add
+// them to the state once (errors as the row walk's; updating the state term by
+// term cost 12 to 22 % more error and saved 5 % of the time).
 #pragma once
 
 #include "kernels.h"
@@ -80,7 +82,7 @@ __global__ void __launch_bounds__(32 * reg_tile(sizeof(R) == 8 ? 0 : 1, BW).warp
   if (ctl->done) return;  // the whole block
   const int lane = threadIdx.x & 31;
   if (threadIdx.x < 2) {
-    LS::consts(C, lane, ctl->dt / ctl->dx[lane], K[lane]);
+    LS::consts(C, lane, dt_over_dx<R>(ctl, lane), K[lane]);
     T[lane] = K[lane];  // transverse terms act on -tau/2
     T[lane].t0 *= R(-0.5);
     T[lane].t1 *= R(-0.5);
@@ -120,16 +122,17 @@ __global__ void __launch_bounds__(32 * reg_tile(sizeof(R) == 8 ? 0 : 1, BW).warp
     }
   };
 
-  // per column: the state less its x updates of rows R-1, R-2; tau_x of rows
+  // per column: the increments of rows R-1, R-2 so far (added to the state once,
+  // when the row is finished, so that they round at their own size); tau_x of rows
   // R-1 .. R-3; y-face strengths of faces R-1, R-2, what face R-2 gives the
   // cell above it; (p, v) of row R-1
-  R acc1[N][M], acc2[N][M], tx1[N], tx2[N], tx3[N], zb1[N][NS], zb2[N][NS], zp2[N][NS];
+  R q1[N][M], q2[N][M], acc1[N][M], acc2[N][M], tx1[N], tx2[N], tx3[N], zb1[N][NS], zb2[N][NS], zp2[N][NS];
   R pz[N], vz[N];
 #pragma unroll
   for (int c = 0; c < N; ++c) {
     tx1[c] = tx2[c] = tx3[c] = pz[c] = vz[c] = R(0);
 #pragma unroll
-    for (int k = 0; k < M; ++k) acc1[c][k] = acc2[c][k] = R(0);
+    for (int k = 0; k < M; ++k) acc1[c][k] = acc2[c][k] = q1[c][k] = q2[c][k] = R(0);
 #pragma unroll
     for (int s = 0; s < NS; ++s) zb1[c][s] = zb2[c][s] = zp2[c][s] = R(0);
   }
@@ -138,11 +141,14 @@ __global__ void __launch_bounds__(32 * reg_tile(sizeof(R) == 8 ? 0 : 1, BW).warp
   if (c0 < nx) load(r0 - 2, qn);
   // (a warp whose strip starts past the grid has nothing to do)
   for (int r = c0 < nx ? r0 - 2 : r1 + 2; r <= r1 + 1; ++r) {
-    R acc0[N][M], tx[N], ty[N], zo[N];
+    R q0[N][M], acc0[N][M], tx[N], ty[N], zo[N];
 #pragma unroll
     for (int c = 0; c < N; ++c) {
 #pragma unroll
-      for (int k = 0; k < M; ++k) acc0[c][k] = qn[c][k];
+      for (int k = 0; k < M; ++k) {
+        q0[c][k] = qn[c][k];
+        acc0[c][k] = R(0);
+      }
       tx[c] = ty[c] = zo[c] = R(0);
     }
     if (r <= r1) load(r + 1, qn);
@@ -150,7 +156,7 @@ __global__ void __launch_bounds__(32 * reg_tile(sizeof(R) == 8 ? 0 : 1, BW).warp
     if (doy) {
 #pragma unroll
       for (int c = 0; c < N; ++c) {
-        const R p = acc0[c][0], v = acc0[c][V];
+        const R p = q0[c][0], v = q0[c][V];
         R zb[NS], up[NS], fp[NS], fm[NS];
         LS::strength(C, pz[c], vz[c], p, v, zb);
 #pragma unroll
@@ -174,13 +180,13 @@ __global__ void __launch_bounds__(32 * reg_tile(sizeof(R) == 8 ? 0 : 1, BW).warp
     if (dox && r >= r0 - 1 && r <= r1) {
       R b[N][NS], fp[N][NS], fm[N + 1][NS], bl[NS], bu[NS];
       {
-        const R pl = __shfl_up_sync(FULL, acc0[N - 1][0], 1);
-        const R ul = VEL ? __shfl_up_sync(FULL, acc0[N - 1][U], 1) : R(0);
-        LS::strength(C, pl, ul, acc0[0][0], acc0[0][U], b[0]);
+        const R pl = __shfl_up_sync(FULL, q0[N - 1][0], 1);
+        const R ul = VEL ? __shfl_up_sync(FULL, q0[N - 1][U], 1) : R(0);
+        LS::strength(C, pl, ul, q0[0][0], q0[0][U], b[0]);
       }
 #pragma unroll
       for (int c = 1; c < N; ++c)
-        LS::strength(C, acc0[c - 1][0], acc0[c - 1][U], acc0[c][0], acc0[c][U], b[c]);
+        LS::strength(C, q0[c - 1][0], q0[c - 1][U], q0[c][0], q0[c][U], b[c]);
 #pragma unroll
       for (int s = 0; s < NS; ++s) {
         bl[s] = __shfl_up_sync(FULL, b[N - 1][s], 1);
@@ -201,8 +207,8 @@ __global__ void __launch_bounds__(32 * reg_tile(sizeof(R) == 8 ? 0 : 1, BW).warp
       for (int c = 0; c < N; ++c) {
         R z;
         LS::cell(fp[c], fm[c + 1], tx[c], z);
-        acc0[c][0] -= tx[c];
-        if (VEL) acc0[c][U] = LS::normal(K[0], acc0[c][U], z);
+        acc0[c][0] = -tx[c];
+        if (VEL) acc0[c][U] = LS::normal(K[0], R(0), z);
         if (!FAST && mode == 1) tx[c] = LS::plain(K[0], b[c], c == N - 1 ? bu : b[c < N - 1 ? c + 1 : 0]);
       }
     }
@@ -224,7 +230,7 @@ __global__ void __launch_bounds__(32 * reg_tile(sizeof(R) == 8 ? 0 : 1, BW).warp
           const bool two = N > 1 && g0 + c + 1 < nx;
 #pragma unroll
           for (int k = 0; k < M; ++k) {
-            const R a = acc2[c][k], b = acc2[c + (N > 1)][k];
+            const R a = q2[c][k] + acc2[c][k], b = q2[c + (N > 1)][k] + acc2[c + (N > 1)][k];
             bad |= not_finite(a);
             if (two) bad |= not_finite(b);
             st_pair(qo + k * plane + (size_t)(r - 2) * nx + (g0 + c), two, vec, a, b);
@@ -241,6 +247,8 @@ __global__ void __launch_bounds__(32 * reg_tile(sizeof(R) == 8 ? 0 : 1, BW).warp
       for (int k = 0; k < M; ++k) {
         acc2[c][k] = acc1[c][k];
         acc1[c][k] = acc0[c][k];
+        q2[c][k] = q1[c][k];
+        q1[c][k] = q0[c][k];
       }
     }
   }

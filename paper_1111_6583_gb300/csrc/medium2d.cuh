@@ -20,8 +20,8 @@
 // same bits.
 //
 // What bounds it: FP32 issue and latency (43 % issue at 1024^2, one wave of
-// 1026 warps), FP64 the FP64 pipe.  1024^2 with capacity FP32 211 -> 37
-// us/step, FP64 973 -> 377 us, 301 x 280 FP64 110 -> 80 us against a record of
+// 1026 warps), FP64 the FP64 pipe.  1024^2 with capacity FP32 211 -> 42
+// us/step, FP64 973 -> 370 us, 301 x 280 FP64 110 -> 81 us against a record of
 // seven vectors per face written by two sweeps and gathered by an update.
 #pragma once
 
@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(32 * reg_tile(sizeof(R) == 8 ? 0 : 1, BW).warp
   MedK<R> K[2];
 #pragma unroll
   for (int d = 0; d < 2; ++d) {
-    K[d].lam = (R)(ctl->dt / ctl->dx[d]);
+    K[d].lam = dt_over_dx<R>(ctl, d);
     K[d].hl = R(0.5) * K[d].lam;
     K[d].hal = C.order == 2 ? (C.lim == CLAW_LIM_MC ? R(1) : R(0.5)) : R(0);
   }
@@ -143,17 +143,18 @@ __global__ void __launch_bounds__(32 * reg_tile(sizeof(R) == 8 ? 0 : 1, BW).warp
     return o;
   };
 
-  // per column: state less its updates (rows r-1, r-2), media of rows r-1, r-2,
+  // per column: increments so far (rows r-1, r-2; added to the state once, when
+  // the row is finished), media of rows r-1, r-2,
   // 1/(Z_l + Z_r) of the lower x-face of row r-1, r-2, tau_x of row r-1;
   // y-faces: strengths of faces r-1, r-2, what face r-2 gives the cell above
-  R acc1[N][M], acc2[N][M], iz1[N], iz2[N], tx1[N], ya1[N][2], ya2[N][2], yp2[N][2], pz[N], vz[N];
+  R q1[N][M], q2[N][M], acc1[N][M], acc2[N][M], iz1[N], iz2[N], tx1[N], ya1[N][2], ya2[N][2], yp2[N][2], pz[N], vz[N];
   Med<R> m1[N], m2[N];
 #pragma unroll
   for (int c = 0; c < N; ++c) {
     iz1[c] = iz2[c] = tx1[c] = pz[c] = vz[c] = R(0);
     m1[c] = m2[c] = Med<R>{R(1), R(0), R(0), R(0), R(0)};
 #pragma unroll
-    for (int k = 0; k < M; ++k) acc1[c][k] = acc2[c][k] = R(0);
+    for (int k = 0; k < M; ++k) acc1[c][k] = acc2[c][k] = q1[c][k] = q2[c][k] = R(0);
 #pragma unroll
     for (int s = 0; s < 2; ++s) ya1[c][s] = ya2[c][s] = yp2[c][s] = R(0);
   }
@@ -162,12 +163,15 @@ __global__ void __launch_bounds__(32 * reg_tile(sizeof(R) == 8 ? 0 : 1, BW).warp
   R qn[N][6];
   if (c0 < nx) load(r0 - 2, qn);
   for (int r = c0 < nx ? r0 - 2 : r1 + 2; r <= r1 + 1; ++r) {
-    R acc0[N][M], tx[N], ty[N], iz[N];
+    R q0[N][M], acc0[N][M], tx[N], ty[N], iz[N];
     Med<R> m0[N];
 #pragma unroll
     for (int c = 0; c < N; ++c) {
 #pragma unroll
-      for (int k = 0; k < M; ++k) acc0[c][k] = qn[c][k];
+      for (int k = 0; k < M; ++k) {
+        q0[c][k] = qn[c][k];
+        acc0[c][k] = R(0);
+      }
       m0[c].c = qn[c][4];
       m0[c].Z = mulr(qn[c][3], qn[c][4]);
       m0[c].cz = mulr(m0[c].c, m0[c].Z);
@@ -183,7 +187,7 @@ __global__ void __launch_bounds__(32 * reg_tile(sizeof(R) == 8 ? 0 : 1, BW).warp
     if (doy) {
 #pragma unroll
       for (int c = 0; c < N; ++c) {
-        const R p = acc0[c][0], v = acc0[c][2];
+        const R p = q0[c][0], v = q0[c][2];
         izy[c] = FM<R>::rcp(m1[c].Z + m0[c].Z);
         R a[2], fp[2], fm[2];
         const R dp = p - pz[c], du = v - vz[c];
@@ -213,14 +217,14 @@ __global__ void __launch_bounds__(32 * reg_tile(sizeof(R) == 8 ? 0 : 1, BW).warp
     if (dox && xrow) {
       R a[N][2], fp[N][2], fm[N + 1][2];
       const Med<R> ml = shup(m0[N - 1]);
-      const R pl = __shfl_up_sync(FULL, acc0[N - 1][0], 1);
-      const R ul = __shfl_up_sync(FULL, acc0[N - 1][1], 1);
+      const R pl = __shfl_up_sync(FULL, q0[N - 1][0], 1);
+      const R ul = __shfl_up_sync(FULL, q0[N - 1][1], 1);
 #pragma unroll
       for (int c = 0; c < N; ++c) {
         const R Zl = c == 0 ? ml.Z : m0[c > 0 ? c - 1 : 0].Z;
         iz[c] = FM<R>::rcp(Zl + m0[c].Z);
-        const R dp = acc0[c][0] - (c == 0 ? pl : acc0[c > 0 ? c - 1 : 0][0]);
-        const R du = acc0[c][1] - (c == 0 ? ul : acc0[c > 0 ? c - 1 : 0][1]);
+        const R dp = q0[c][0] - (c == 0 ? pl : q0[c > 0 ? c - 1 : 0][0]);
+        const R du = q0[c][1] - (c == 0 ? ul : q0[c > 0 ? c - 1 : 0][1]);
         a[c][0] = mulr(fma(m0[c].Z, du, -dp), iz[c]);
         a[c][1] = mulr(fma(Zl, du, dp), iz[c]);
       }
@@ -241,8 +245,8 @@ __global__ void __launch_bounds__(32 * reg_tile(sizeof(R) == 8 ? 0 : 1, BW).warp
       for (int c = 0; c < N; ++c) {
         const R li = mulr(K[0].lam, m0[c].ik);
         tx[c] = mulr(li, fp[c][0] + fm[c + 1][0]);
-        acc0[c][0] -= tx[c];
-        acc0[c][1] = fma(-li, fp[c][1] + fm[c + 1][1], acc0[c][1]);
+        acc0[c][0] = -tx[c];
+        acc0[c][1] = mulr(-li, fp[c][1] + fm[c + 1][1]);
         if (!FAST && mode == 1)
           tx[c] = mulr(li, fma(m0[c].cz, a[c][1], mulr(m0[c].cz, c == N - 1 ? bu : a[c < N - 1 ? c + 1 : 0][0])));
       }
@@ -291,7 +295,7 @@ __global__ void __launch_bounds__(32 * reg_tile(sizeof(R) == 8 ? 0 : 1, BW).warp
           const bool two = N > 1 && g0 + c + 1 < nx;
 #pragma unroll
           for (int k = 0; k < M; ++k) {
-            const R a = acc2[c][k], b = acc2[c + (N > 1)][k];
+            const R a = q2[c][k] + acc2[c][k], b = q2[c + (N > 1)][k] + acc2[c + (N > 1)][k];
             bad |= not_finite(a);
             if (two) bad |= not_finite(b);
             st_pair(qo + k * plane + (size_t)(r - 2) * nx + (g0 + c), two, vec, a, b);
@@ -310,6 +314,8 @@ __global__ void __launch_bounds__(32 * reg_tile(sizeof(R) == 8 ? 0 : 1, BW).warp
       for (int k = 0; k < M; ++k) {
         acc2[c][k] = acc1[c][k];
         acc1[c][k] = acc0[c][k];
+        q2[c][k] = q1[c][k];
+        q1[c][k] = q0[c][k];
       }
     }
   }
