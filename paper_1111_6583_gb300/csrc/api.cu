@@ -48,6 +48,17 @@ KernelSet kernels_for(int rp, int nd, int prec) {
   return KernelSet{};
 }
 
+KernelSet kernels_for(const claw_method& m, int nd) {
+  KernelSet ks = kernels_for(m.rp, nd, m.prec);
+  // FP32 van Leer runs the row walk for the systems that have both kernels
+  if (ks.valid && m.prec == CLAW_FP32 && m.lim == CLAW_LIM_VANLEER && ks.tx64_walk) {
+    ks.tx64 = ks.tx64_walk;
+    ks.tx128 = ks.tx128_walk;
+    ks.reg_kernel = 0;
+  }
+  return ks;
+}
+
 template <typename R>
 void fill_consts(const claw_method& m, MConsts<R>& C) {
   std::memset(&C, 0, sizeof(C));
@@ -788,7 +799,7 @@ claw_status claw_solver_create(const claw_method* m, const claw_grid* g, void* s
   *out = nullptr;
   if (const char* why = check_grid(*g, *m)) return fail(nullptr, why);
   if (const char* why = check_method(*m, g->ndim)) return fail(nullptr, why);
-  KernelSet ks = kernels_for(m->rp, g->ndim, m->prec);
+  KernelSet ks = kernels_for(*m, g->ndim);
   if (!ks.valid) return fail(nullptr, "no kernels for this solver/dimension/precision");
   claw_solver* s = new claw_solver();
   s->m = *m;
@@ -1258,7 +1269,7 @@ claw_status claw_batch_create(const claw_method* m, const claw_grid* grids, int 
     if (grids[k].ndim != nd) return bfail(nullptr, "all members need the same ndim");
   }
   if (const char* why = check_method(*m, nd)) return bfail(nullptr, why);
-  KernelSet ks = kernels_for(m->rp, nd, m->prec);
+  KernelSet ks = kernels_for(*m, nd);
   if (!ks.valid) return bfail(nullptr, "no kernels for this solver/dimension/precision");
   claw_batch* b = new claw_batch();
   b->m = *m;
@@ -1665,7 +1676,7 @@ claw_status claw_server_create_nd(const claw_method* m, int ndim, size_t hbm_bud
   const int nd = ndim;
   if (const char* why = check_method(*m, nd)) return sfail(nullptr, why);
   const int faces = on_faces(*m, nd);
-  KernelSet ks = kernels_for(m->rp, nd, m->prec);
+  KernelSet ks = kernels_for(*m, nd);
   if (!ks.valid) return sfail(nullptr, "no kernels for this solver/dimension/precision");
   claw_server* v = new claw_server();
   v->m = *m;

@@ -53,6 +53,7 @@ struct KernelSet {
   launch_fn source;        // axisymmetric Euler source step (2D Euler systems)
   int max_bw;              // 2D classic: widest block whose static shared memory fits
   int tx64, tx128;         // 2D classic: columns of a tile at either width
+  int tx64_walk, tx128_walk;  // ... of the row walk, for systems that also run it (else 0)
   int reg_kernel;          // 2D classic: register-resident kernel (chunks of 2 rows pay)
   int (*blocks3)(int nx, int ny, int nz);  // 3D: blocks of an attempt (they count the arrivals)
   int sharp_shapes;        // 2D SharpClaw WENO5: bit i set when tile kSharpShapes2[i]

@@ -8,7 +8,10 @@
 #include "kernels.h"
 #include "linear2d.cuh"
 #include "medium2d.cuh"
+#include "roe2d.cuh"
 #include "sharpclaw.cuh"
+
+#include <type_traits>
 
 namespace claw {
 
@@ -180,6 +183,16 @@ inline bool uses_faces(int capa) {
   return ND <= 2 && capa >= 0 && !medium_kernel<RP, ND>();
 }
 
+// systems whose 2D step runs roe2d_kernel
+template <class RP>
+struct is_roe2d {
+  static constexpr bool value = false;
+};
+template <typename R>
+struct is_roe2d<RpSW<R, 2>> {
+  static constexpr bool value = true;
+};
+
 template <class RP, typename R, int ND>
 struct Launchers {
   static cudaError_t classic(const LaunchArgs& a) {
@@ -231,7 +244,7 @@ struct Launchers {
       // systems of up to three fields: with more, the two block widths of the
       // fixed-settings form were seen to round differently, and every tile
       // shape must give the same bits
-      if ((sizeof(R) == 4 || is_linear_rp<RP, R>::value) && RP::M <= 3 && C.lim == CLAW_LIM_MC && C.order == 2 &&
+      if ((sizeof(R) == 4 || is_linear_rp<RP, R>::value || is_roe2d<RP>::value) && RP::M <= 3 && C.lim == CLAW_LIM_MC && C.order == 2 &&
           C.transverse == 2 && a.sweep == 0)
         return classic2d<true>(a, C);
       return classic2d<false>(a, C);
@@ -244,6 +257,22 @@ struct Launchers {
     const int threads = 32 * reg_tile(sizeof(R) == 8 ? 0 : 1, a.bw).warps;
     kern<<<launch_grid(a.ntiles_total), threads, 0, a.stream>>>(a.members, a.tiles, C, a.h, a.sweep);
     return cudaGetLastError();
+  }
+  template <bool FAST>
+  static cudaError_t roe2d(const LaunchArgs& a, const MConsts<R>& C) {
+    if constexpr (ND == 2 && is_roe2d<RP>::value) {
+      constexpr int prec = sizeof(R) == 8 ? 0 : 1;
+      using V = typename std::conditional<sizeof(R) == 8, double, F2>::type;
+      auto go = [&](auto kern, int threads) {
+        kern<<<launch_grid(a.ntiles_total), threads, 0, a.stream>>>(a.members, a.tiles, C, a.h,
+                                                                   a.sweep);
+        return cudaGetLastError();
+      };
+      constexpr int w64 = roe_tile(prec, 64).warps, w128 = roe_tile(prec, 128).warps;
+      if (a.bw == 128) return go(roe2d_kernel<RP, V, w128, FAST>, 32 * w128);
+      if (a.bw == 64) return go(roe2d_kernel<RP, V, w64, FAST>, 32 * w64);
+    }
+    return cudaErrorInvalidValue;
   }
   // FAST (FP32 only): the common settings fixed at compile time
   template <bool FAST>
@@ -289,12 +318,18 @@ struct Launchers {
   }
   template <bool FAST>
   static cudaError_t classic2d(const LaunchArgs& a, const MConsts<R>& C) {
+    if constexpr (ND == 2 && is_roe2d<RP>::value) {
+      // FP32 van Leer stays on the row walk: where strengths underflow its
+      // ratio ends a run as non-finite, and which runs end so stays as it was
+      if (sizeof(R) == 8 || C.lim != CLAW_LIM_VANLEER) return roe2d<FAST>(a, C);
+    }
     if constexpr (ND == 2 && is_linear_rp<RP, R>::value) {
       // bits do not depend on FAST or on the width (explicit rounding)
       if (a.bw == 128) return reg2d(linear2d_kernel<RP, R, 128, FAST>, a, C);
       if (a.bw == 64) return reg2d(linear2d_kernel<RP, R, 64, FAST>, a, C);
       return cudaErrorInvalidValue;
-    } else if constexpr (ND == 2 && RP::MA == 0 && (!FAST || (sizeof(R) == 4 && RP::M <= 3))) {
+    } else if constexpr (ND == 2 && RP::MA == 0 && (!FAST || (sizeof(R) == 4 && RP::M <= 3)) &&
+                         (!is_roe2d<RP>::value || (sizeof(R) == 4 && !FAST))) {
       if constexpr (classic2d_fits<RP, R>(128)) {
         if (a.bw == 128) {
           classic2d_kernel<RP, R, 128, FAST><<<launch_grid(a.ntiles_total), 128, 0, a.stream>>>(
@@ -426,10 +461,13 @@ KernelSet make_set(bool has_char) {
   k.source = &Launchers<RP, R, ND>::source;
   k.blocks3 = &Launchers<RP, R, ND>::blocks3;
   k.max_bw = classic2d_fits<RP, R>(128) ? 128 : 64;
-  k.reg_kernel = ND == 2 && (is_linear_rp<RP, R>::value || medium_kernel<RP, ND>());
+  constexpr bool roe = ND == 2 && is_roe2d<RP>::value;
+  k.reg_kernel = ND == 2 && (is_linear_rp<RP, R>::value || medium_kernel<RP, ND>() || roe);
   constexpr int prec = sizeof(R) == 8 ? 0 : 1;
-  k.tx64 = k.reg_kernel ? reg_tile(prec, 64).tx : 64 - 4;
-  k.tx128 = k.reg_kernel ? reg_tile(prec, 128).tx : 128 - 4;
+  k.tx64 = roe ? roe_tile(prec, 64).tx : k.reg_kernel ? reg_tile(prec, 64).tx : 64 - 4;
+  k.tx128 = roe ? roe_tile(prec, 128).tx : k.reg_kernel ? reg_tile(prec, 128).tx : 128 - 4;
+  k.tx64_walk = roe ? 64 - 4 : 0;
+  k.tx128_walk = roe ? 128 - 4 : 0;
   constexpr size_t lim = kSmemPerBlock;
   k.sharp_shapes = (sharp_smem_bytes<RP, R, 2, 16, 8, 3>() <= lim ? 1 : 0) |
                    (sharp_smem_bytes<RP, R, 2, 32, 4, 3>() <= lim ? 2 : 0) |

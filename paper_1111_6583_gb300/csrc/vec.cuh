@@ -47,7 +47,11 @@ __device__ __forceinline__ F2 vmul(F2 a, F2 b) {
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
   return r;
 }
-__device__ __forceinline__ F2 vsub(F2 a, F2 b) { return vfma(F2(-1.f), b, a); }
+__device__ __forceinline__ F2 vsub(F2 a, F2 b) {
+  F2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
 template <typename R>
 __device__ __forceinline__ R vfma(R a, R b, R c) { return fma(a, b, c); }
 template <typename R>
@@ -58,6 +62,11 @@ __device__ __forceinline__ R vsub(R a, R b) { return a - b; }
 // every instantiation rounds alike
 __device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double vmul(double a, double b) { return __dmul_rn(a, b); }
+
+// c - a b
+__device__ __forceinline__ F2 vnfma(F2 a, F2 b, F2 c) { return vsub(c, vmul(a, b)); }
+template <typename R>
+__device__ __forceinline__ R vnfma(R a, R b, R c) { return fma(-a, b, c); }
 
 // f on each value (pairs: on both halves)
 template <class F>
@@ -117,17 +126,14 @@ __device__ __forceinline__ V vrsq(V a) {
   using S = typename VecOf<V>::S;
   return vmap([](S x) { return FM<S>::rsqrt(x); }, a);
 }
-// the negative part of a (a itself where a < 0, else 0)
+// v where s < 0 (m) and elsewhere (p), 0 in the other one.  FP64 by selects
+// (the FP64 pipe is the scarce unit), pairs by one packed subtraction
 template <class V>
-__device__ __forceinline__ V vneg_part(V a) {
+__device__ __forceinline__ void vsplit(V s, V v, V& m, V& p) {
   using S = typename VecOf<V>::S;
-  return vmap([](S x) { return lt0(x) ? x : S(0); }, a);
-}
-// v where s < 0, else 0
-template <class V>
-__device__ __forceinline__ V vwhere_neg(V s, V v) {
-  using S = typename VecOf<V>::S;
-  return vmap([](S a, S x) { return lt0(a) ? x : S(0); }, s, v);
+  m = vmap([](S a, S x) { return lt0(a) ? x : S(0); }, s, v);
+  if constexpr (VecOf<V>::N == 1) p = lt0(s) ? S(0) : v;
+  else p = vsub(v, m);
 }
 
 // the value of the column to the left / right (columns run over a warp's
