@@ -523,6 +523,7 @@ struct claw_solver {
   int npart = 0;
   int ntiles = 0, bw = 128, h = 32;
   int tuned = 0;
+  int mode1d = 0;  // 1D: the caller set a work mode
   void* work3 = nullptr;  // per-face path: face arrays
   size_t work3_bytes = 0;
   cudaGraphExec_t gexec = nullptr;
@@ -575,6 +576,23 @@ cudaError_t solver_attempt(claw_solver* s, cudaStream_t st) {
                         s->work3, s->work3_bytes);
 }
 
+// small 1D grids take several attempts per launch (unless the caller chose a
+// work mode)
+bool multi1d(const claw_solver* s) {
+  return s->nd == 1 && s->m.scheme == CLAW_CLASSIC && !s->faces && !s->mode1d &&
+         cluster1d_fits(s->g.n[0], s->prec, s->ks.MA, s->ks.linear);
+}
+cudaError_t solver_attempts(claw_solver* s, int n, cudaStream_t st) {
+  if (n > 0 && multi1d(s)) {
+    LaunchArgs a{s->d_mem, nullptr, s->ntiles, s->consts.data(), 0, 0, 0, st};
+    a.attempts = n;
+    return s->ks.multi1d(a);
+  }
+  cudaError_t e = cudaSuccess;
+  for (int i = 0; i < n && e == cudaSuccess; ++i) e = solver_attempt(s, st);
+  return e;
+}
+
 cudaError_t read_ctl(claw_solver* s) {
   cudaError_t e = cudaMemcpyAsync(s->h_ctl, s->d_ctl, sizeof(DevCtl), cudaMemcpyDeviceToHost, s->st);
   if (e != cudaSuccess) return e;
@@ -597,7 +615,7 @@ cudaError_t build_graph(claw_solver* s, int k) {
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamBeginCapture(s->st, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return e;
-  for (int i = 0; i < k && e == cudaSuccess; ++i) e = solver_attempt(s, s->st);
+  e = solver_attempts(s, k, s->st);
   cudaError_t e2 = cudaStreamEndCapture(s->st, &g);
   if (e != cudaSuccess) {
     if (g) cudaGraphDestroy(g);
@@ -896,6 +914,7 @@ claw_status claw_solver_tune(claw_solver* s, int mode, int* bw, int* h) {
     if (s->m.scheme == CLAW_CLASSIC && s->nd == 1 && h &&
         (*h == kWork1dTiles || *h == kWork1dUnits)) {
       s->h = *h;
+      s->mode1d = 1;
       s->tuned = 1;
       drop_graph(s);
       if (bw) *bw = s->bw;
@@ -933,7 +952,7 @@ claw_status claw_advance(claw_solver* s, int n) {
   if (!s || !s->bound) return fail(s, "solver not bound");
   if (n < 0) return fail(s, "n must be >= 0");
   SCK(enter(s));
-  for (int i = 0; i < n; ++i) SCK(solver_attempt(s, s->st));
+  SCK(solver_attempts(s, n, s->st));
   SCK(leave(s));
   return CLAW_OK;
 }
@@ -962,7 +981,7 @@ claw_status claw_evolve_to_time(claw_solver* s, double t_end, int64_t max_steps,
                                 claw_step_info* info) {
   if (!s || !s->bound) return fail(s, "solver not bound");
   SCK(enter(s));
-  if (!s->tuned) SCK(autotune(s));
+  if (!s->tuned && !multi1d(s)) SCK(autotune(s));
   SCK(launch_set_t_end(s->d_ctl, 1, t_end, (long long)max_steps, s->st));
   const int GK = 16;
   if (use_graph && s->gk != GK) SCK(build_graph(s, GK));
@@ -981,7 +1000,7 @@ claw_status claw_evolve_to_time(claw_solver* s, double t_end, int64_t max_steps,
       for (long long r = 0; r < reps; ++r) SCK(cudaGraphLaunch(s->gexec, s->st));
       launched += reps * GK;
     } else {
-      for (long long i = 0; i < k; ++i) SCK(solver_attempt(s, s->st));
+      SCK(solver_attempts(s, (int)k, s->st));
       launched += k;
     }
     if (launched > (1LL << 40)) return fail(s, "evolve made no progress");
@@ -1118,7 +1137,7 @@ claw_status claw_step_host(claw_solver* s, const void* q_host_in, void* q_host_o
   SCK(enter(s));
   SCK(cudaMemcpyAsync(s->q_user, q_host_in, s->sbytes, cudaMemcpyHostToDevice, s->st));
   SCK(launch_reset_cur(s->d_ctl, s->st));
-  for (int i = 0; i < n; ++i) SCK(solver_attempt(s, s->st));
+  SCK(solver_attempts(s, n, s->st));
   // the slot that holds the result when every attempt is accepted; a device
   // copy moves the result there otherwise, so both reads queue behind the
   // attempts with one synchronisation at the end

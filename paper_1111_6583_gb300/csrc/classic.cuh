@@ -11,8 +11,11 @@
 // tiles) runs the controller.
 #pragma once
 
+#include <cooperative_groups.h>
+
 #include "async_copy.cuh"
 #include "kernels.h"
+#include "linear.cuh"
 #include "riemann.cuh"
 
 namespace claw {
@@ -42,6 +45,11 @@ template <typename R, int K>
 struct VecIO;
 template <>
 struct VecIO<float, 4> {
+  // past L1: values that other blocks of the same launch wrote
+  __device__ static __forceinline__ void load_l2(const float* p, float (&v)[4]) {
+    const float4 a = __ldcg((const float4*)p);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+  }
   // from a 16-byte aligned shared-memory slot
   __device__ static __forceinline__ void load_shared(const float* p, float (&v)[4]) {
     const float4 a = *(const float4*)p;
@@ -57,6 +65,12 @@ struct VecIO<float, 4> {
 };
 template <>
 struct VecIO<float, 8> {
+  // past L1: values that other blocks of the same launch wrote
+  __device__ static __forceinline__ void load_l2(const float* p, float (&v)[8]) {
+    const float4 a = __ldcg((const float4*)p), b = __ldcg((const float4*)p + 1);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+  }
   // from a 16-byte aligned shared-memory slot
   __device__ static __forceinline__ void load_shared(const float* p, float (&v)[8]) {
     const float4 a = ((const float4*)p)[0], b = ((const float4*)p)[1];
@@ -75,6 +89,11 @@ struct VecIO<float, 8> {
 };
 template <>
 struct VecIO<double, 2> {
+  // past L1: values that other blocks of the same launch wrote
+  __device__ static __forceinline__ void load_l2(const double* p, double (&v)[2]) {
+    const double2 a = __ldcg((const double2*)p);
+    v[0] = a.x; v[1] = a.y;
+  }
   // from a 16-byte aligned shared-memory slot
   __device__ static __forceinline__ void load_shared(const double* p, double (&v)[2]) {
     const double2 a = *(const double2*)p;
@@ -220,6 +239,204 @@ __device__ __forceinline__ void limit1d(const MConsts<R>& C, int order,
   correction<RP, R, 0, LIMC>(C, Wc, sc, dot, nrm, dtdx, F);
 }
 
+template <class RP, typename R>
+struct is_elasticity1d {
+  static constexpr bool value = false;
+};
+template <typename R>
+struct is_elasticity1d<RpElasticity<R, 1>, R> {
+  static constexpr bool value = true;
+};
+
+// The arithmetic of one warp unit: lane l holds cells qa (aux aa) at and above
+// its interface 0; returns the new values of its cells (those of lanes 0 and
+// 31 are incomplete).  faces: the lane's interfaces up to the grid's last one.
+// Constant-coefficient linear systems and the f-wave elasticity solver in
+// strength form (as linear.cuh): a third to two thirds of the operations of
+// the wave-vector form, and explicit rounding.
+template <class RP, typename R, int K, bool FAST, int MAS>
+__device__ __forceinline__ void unit1d(const MConsts<R>& C, int order, R dtdx, const LinK<R>& lk,
+                                       const R (&qa)[K][RP::M], const R (&aa)[K][MAS], int lane,
+                                       int faces, R (&qout)[K][RP::M], R& smax) {
+  constexpr int M = RP::M, MW = RP::MW;
+  constexpr int LIMC = FAST ? CLAW_LIM_MC : -1;
+  constexpr unsigned FULL = 0xffffffffu;
+  if constexpr (is_linear_rp<RP, R>::value) {
+    using LS = Lin<RP, R>;
+    constexpr int NS = LS::NS, U = LS::VEL ? 1 : 0;
+    R b[K][NS], fp[K][NS], fm[K + 1][NS], bl[NS], bu[NS];
+    {
+      const R pl = __shfl_up_sync(FULL, qa[K - 1][0], 1);
+      const R ul = LS::VEL ? __shfl_up_sync(FULL, qa[K - 1][U], 1) : R(0);
+      LS::strength(C, pl, ul, qa[0][0], qa[0][U], b[0]);
+    }
+#pragma unroll
+    for (int c = 1; c < K; ++c)
+      LS::strength(C, qa[c - 1][0], qa[c - 1][U], qa[c][0], qa[c][U], b[c]);
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      bl[s] = __shfl_up_sync(FULL, b[K - 1][s], 1);
+      bu[s] = __shfl_down_sync(FULL, b[0][s], 1);
+    }
+#pragma unroll
+    for (int c = 0; c < K; ++c) {
+      R up[NS];
+#pragma unroll
+      for (int s = 0; s < NS; ++s)
+        up[s] = LS::upwind(lk, s, c == 0 ? bl[s] : b[c > 0 ? c - 1 : 0][s],
+                           c == K - 1 ? bu[s] : b[c < K - 1 ? c + 1 : 0][s]);
+      LS::template face<FAST>(lk, C.lim, b[c], up, fp[c], fm[c]);
+    }
+#pragma unroll
+    for (int s = 0; s < NS; ++s) fm[K][s] = __shfl_down_sync(FULL, fm[0][s], 1);
+#pragma unroll
+    for (int c = 0; c < K; ++c) {
+      R tau, zo;
+      LS::cell(fp[c], fm[c + 1], tau, zo);
+      qout[c][0] = qa[c][0] - tau;
+      if (LS::VEL) qout[c][U] = LS::normal(lk, qa[c][U], zo);
+    }
+    smax = LS::speed(C, 0);
+    return;
+  }
+  if constexpr (is_elasticity1d<RP, R>::value) {
+    // f-waves b_1 (1, Z_l) and b_2 (1, -Z_r): theta_1 is the ratio of strengths
+    // times (1 + Z_l Z_r) / (1 + Z_l^2) (theta_2: 1 + Z_r^2), since the upwind
+    // face of either shares a cell with this one.  FP32 van Leer takes the
+    // wave-vector form below.
+    if (sizeof(R) == 8 || FAST || C.lim != CLAW_LIM_VANLEER) {
+      using CP = CellPrep<RP, R>;
+      const R hal = order == 2 ? ((FAST || C.lim == CLAW_LIM_MC) ? R(1) : R(0.5)) : R(0);
+      typename CP::Cell pc[K], left;
+      R wn[K], tc[K], lw, lt;  // 1 / (1 + Z^2), hal (1 - dt/dx c) per cell
+#pragma unroll
+      for (int c = 0; c < K; ++c) {
+        CP::prep(C, qa[c], aa[c], pc[c]);
+        wn[c] = FM<R>::rcp(fma(pc[c].Z, pc[c].Z, R(1)));
+        tc[c] = fma(-hal * dtdx, pc[c].c, hal);
+      }
+      left.e = __shfl_up_sync(FULL, pc[K - 1].e, 1);
+      left.u = __shfl_up_sync(FULL, pc[K - 1].u, 1);
+      left.c = __shfl_up_sync(FULL, pc[K - 1].c, 1);
+      left.Z = __shfl_up_sync(FULL, pc[K - 1].Z, 1);
+      lw = __shfl_up_sync(FULL, wn[K - 1], 1);
+      lt = __shfl_up_sync(FULL, tc[K - 1], 1);
+      R b1[K], b2[K], g[K], p0[K], p1[K], m0[K + 1], m1[K + 1];
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        const R Zl = k ? pc[k > 0 ? k - 1 : 0].Z : left.Z, Zr = pc[k].Z;
+        const R d1 = (k ? pc[k > 0 ? k - 1 : 0].u : left.u) - pc[k].u;
+        const R d2 = (k ? pc[k > 0 ? k - 1 : 0].e : left.e) - pc[k].e;
+        const R iz = FM<R>::rcp(Zl + Zr);
+        b1[k] = mulr(fma(Zr, d1, d2), iz);
+        b2[k] = mulr(fma(Zl, d1, -d2), iz);
+        g[k] = fma(Zl, Zr, R(1));
+      }
+      const R bu = __shfl_down_sync(FULL, b1[0], 1), bl = __shfl_up_sync(FULL, b2[K - 1], 1);
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        const R Zl = k ? pc[k > 0 ? k - 1 : 0].Z : left.Z, Zr = pc[k].Z;
+        const R u1 = mulr(mulr(k < K - 1 ? b1[k < K - 1 ? k + 1 : 0] : bu, g[k]), k ? wn[k > 0 ? k - 1 : 0] : lw);
+        const R u2 = mulr(mulr(k ? b2[k > 0 ? k - 1 : 0] : bl, g[k]), wn[k]);
+        const R T1 = mulr(k ? tc[k > 0 ? k - 1 : 0] : lt, lin_limit<FAST>(C.lim, u1, b1[k]));
+        const R T2 = mulr(tc[k], lin_limit<FAST>(C.lim, u2, b2[k]));
+        const R X1 = b1[k] - T1, X2 = b2[k] - T2;
+        m0[k] = X1 + T2;
+        m1[k] = fma(Zl, X1, -mulr(Zr, T2));
+        p0[k] = X2 + T1;
+        p1[k] = fma(Zl, T1, -mulr(Zr, X2));
+      }
+      m0[K] = __shfl_down_sync(FULL, m0[0], 1);
+      m1[K] = __shfl_down_sync(FULL, m1[0], 1);
+      const int nsp = min(lane == 0 ? 0 : (lane == 31 ? 1 : K), faces);
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        qout[k][0] = fma(-dtdx, p0[k] + m0[k + 1], qa[k][0]);
+        qout[k][1] = fma(-dtdx, p1[k] + m1[k + 1], qa[k][1]);
+        if (k < nsp) {
+          const R a = k ? pc[k > 0 ? k - 1 : 0].c : left.c;
+          if constexpr (sizeof(R) == 4) smax = fmaxf(smax, fmaxf(a, pc[k].c));
+          else smax = nanmax(nanmax(smax, a), pc[k].c);
+        }
+      }
+      return;
+    }
+  }
+  if constexpr (!is_linear_rp<RP, R>::value) {
+    using CP = CellPrep<RP, R>;
+    using Cell = typename CP::Cell;
+    constexpr int NCR = sizeof(Cell) / sizeof(R);
+    static_assert(NCR * sizeof(R) == sizeof(Cell), "Cell holds values of type R only");
+    // each cell prepared once; interface k lies between cells k-1 and k
+    // (global index g0+k), its left cell from the lane below
+    Cell pc[K];
+#pragma unroll
+    for (int c = 0; c < K; ++c) CP::prep(C, qa[c], aa[c], pc[c]);
+    Cell left;
+    {
+      const R* a = reinterpret_cast<const R*>(&pc[K - 1]);
+      R* b = reinterpret_cast<R*>(&left);
+#pragma unroll
+      for (int i = 0; i < NCR; ++i) b[i] = __shfl_up_sync(FULL, a[i], 1);
+    }
+    R W[K][MW][M], s[K][MW], am[K][M], ap[K][M];
+    CP::solve(C, left, pc[0], W[0], s[0], am[0], ap[0]);
+#pragma unroll
+    for (int k = 1; k < K; ++k) CP::solve(C, pc[k - 1], pc[k], W[k], s[k], am[k], ap[k]);
+
+    // max speed over the unit's interfaces that bound cells of the grid: lanes
+    // 1..30 their K, lane 31 its first, lane 0 none
+    const int nsp = min(lane == 0 ? 0 : (lane == 31 ? 1 : K), faces);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      if (k < nsp) {
+#pragma unroll
+        for (int p = 0; p < MW; ++p) {
+          // FP32: a non-finite speed makes the results non-finite too, and
+          // the finiteness sum below reports those, so a plain max will do
+          if constexpr (sizeof(R) == 4) smax = fmaxf(smax, fabsf(s[k][p]));
+          else smax = nanmax(smax, (R)fabs(s[k][p]));
+        }
+      }
+    }
+
+    // waves of interface -1 (lane below) and K (lane above)
+    R Wm[MW][M], Wp[MW][M], sp[MW], amK[M];
+#pragma unroll
+    for (int p = 0; p < MW; ++p) {
+#pragma unroll
+      for (int k = 0; k < M; ++k) {
+        Wm[p][k] = __shfl_up_sync(FULL, W[K - 1][p][k], 1);
+        Wp[p][k] = __shfl_down_sync(FULL, W[0][p][k], 1);
+      }
+      sp[p] = __shfl_down_sync(FULL, s[0][p], 1);
+    }
+#pragma unroll
+    for (int k = 0; k < M; ++k) amK[k] = __shfl_down_sync(FULL, am[0][k], 1);
+
+    // limit interfaces 0..K-1 (F of interface K comes from the lane above)
+    // and update each cell once both of its interfaces are limited:
+    // Q_c - dt/dx [(A+dQ - F)_{c-1/2} + (A-dQ + F)_{c+1/2}]
+    R Fl[M], FK[M];
+    limit1d<RP, R, LIMC>(C, order, Wm, W[0], s[0], K > 1 ? W[1] : Wp, dtdx, Fl);
+#pragma unroll
+    for (int k = 0; k < M; ++k) FK[k] = __shfl_down_sync(FULL, Fl[k], 1);
+#pragma unroll
+    for (int c = 1; c < K; ++c) {
+      R Fr[M];
+      limit1d<RP, R, LIMC>(C, order, W[c - 1], W[c], s[c], c + 1 < K ? W[c + 1] : Wp, dtdx, Fr);
+#pragma unroll
+      for (int k = 0; k < M; ++k) {
+        qout[c - 1][k] = qa[c - 1][k] - dtdx * ((ap[c - 1][k] - Fl[k]) + (am[c][k] + Fr[k]));
+        Fl[k] = Fr[k];
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < M; ++k)
+      qout[K - 1][k] = qa[K - 1][k] - dtdx * ((ap[K - 1][k] - Fl[k]) + (amK[k] + FK[k]));
+  }
+}
+
 // Shared-memory ring of the staged form: per warp S slots, each holding the
 // 32 K cells of every field (and aux field) that one warp unit reads, and one
 // barrier per slot.
@@ -243,8 +460,7 @@ template <class RP, typename R, int NT, int K, int SPW, bool FAST = false, int S
 __global__ void __launch_bounds__(NT, (sizeof(R) == 4 && RP::M <= 2) ? (K >= 8 ? 4 : 8) : 1)
     classic1d_kernel(const Member* __restrict__ members, const Tile* __restrict__ tiles,
                      int ntiles_total, const MConsts<R> C) {
-  constexpr int M = RP::M, MW = RP::MW, MA = RP::MA;
-  constexpr int LIMC = FAST ? CLAW_LIM_MC : -1;
+  constexpr int M = RP::M, MA = RP::MA;
   const int order = FAST ? 2 : C.order;
   constexpr int MAS = MA > 0 ? MA : 1;
   constexpr int NW = NT / 32;      // warp units per tile
@@ -254,19 +470,9 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 && RP::M <= 2) ? (K >= 8 ?
   static_assert(K >= 2, "two or more cells per lane");
   constexpr int T = NW * WC;       // cells per tile
   constexpr unsigned FULL = 0xffffffffu;
-  using CP = CellPrep<RP, R>;
-  using Cell = typename CP::Cell;
-  constexpr int NCR = sizeof(Cell) / sizeof(R);
-  static_assert(NCR * sizeof(R) == sizeof(Cell), "Cell holds values of type R only");
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;  // warp in block
-  // Launched as a programmatic dependent of the previous attempt (single-unit
-  // launches of small grids): wait until that launch has completed and its
-  // memory is visible, then let the next attempt's launch begin (its blocks
-  // wait here in turn), so that launch latency overlaps this attempt.  For a
-  // launch without the attribute both return at once.
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  pdl_enter();
 
   // staged form: the ring, and the warp's producer cursor (the consumer's
   // sequence of units, walked up to S units ahead)
@@ -374,6 +580,8 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 && RP::M <= 2) ? (K >= 8 ?
     if (t0 + sub0 * WC >= nx) continue;
     const int cur = ctl->cur, nbuf = ctl->nbuf;
     const R dtdx = dt_over_dx<R>(ctl, 0);
+    LinK<R> lk{};
+    if constexpr (is_linear_rp<RP, R>::value) Lin<RP, R>::consts(C, 0, dtdx, lk);
     const R* __restrict__ q = (const R*)mb.q[cur];
     R* __restrict__ qo = (R*)mb.q[(cur + 1) % nbuf];
     const R* __restrict__ aux = (const R*)mb.aux;
@@ -481,73 +689,8 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 && RP::M <= 2) ? (K >= 8 ?
         }
       }
 
-      // each cell prepared once; interface k lies between cells k-1 and k
-      // (global index g0+k), its left cell from the lane below
-      Cell pc[K];
-#pragma unroll
-      for (int c = 0; c < K; ++c) CP::prep(C, qa[c], aa[c], pc[c]);
-      Cell left;
-      {
-        const R* a = reinterpret_cast<const R*>(&pc[K - 1]);
-        R* b = reinterpret_cast<R*>(&left);
-#pragma unroll
-        for (int i = 0; i < NCR; ++i) b[i] = __shfl_up_sync(FULL, a[i], 1);
-      }
-      R W[K][MW][M], s[K][MW], am[K][M], ap[K][M];
-      CP::solve(C, left, pc[0], W[0], s[0], am[0], ap[0]);
-#pragma unroll
-      for (int k = 1; k < K; ++k) CP::solve(C, pc[k - 1], pc[k], W[k], s[k], am[k], ap[k]);
-
-      // max speed over the unit's interfaces ustart .. ustart+WC that are
-      // <= nx: lanes 1..30 their K, lane 31 its first, lane 0 none
-      const int nsp = min(lane == 0 ? 0 : (lane == 31 ? 1 : K), nx + 1 - g0);
-#pragma unroll
-      for (int k = 0; k < K; ++k) {
-        if (k < nsp) {
-#pragma unroll
-          for (int p = 0; p < MW; ++p) {
-            // FP32: a non-finite speed makes the results non-finite too, and
-            // the finiteness sum below reports those, so a plain max will do
-            if constexpr (sizeof(R) == 4) smax = fmaxf(smax, fabsf(s[k][p]));
-            else smax = nanmax(smax, (R)fabs(s[k][p]));
-          }
-        }
-      }
-
-      // waves of interface -1 (lane below) and K (lane above)
-      R Wm[MW][M], Wp[MW][M], sp[MW], amK[M];
-#pragma unroll
-      for (int p = 0; p < MW; ++p) {
-#pragma unroll
-        for (int k = 0; k < M; ++k) {
-          Wm[p][k] = __shfl_up_sync(FULL, W[K - 1][p][k], 1);
-          Wp[p][k] = __shfl_down_sync(FULL, W[0][p][k], 1);
-        }
-        sp[p] = __shfl_down_sync(FULL, s[0][p], 1);
-      }
-#pragma unroll
-      for (int k = 0; k < M; ++k) amK[k] = __shfl_down_sync(FULL, am[0][k], 1);
-
-      // limit interfaces 0..K-1 (F of interface K comes from the lane above)
-      // and update each cell once both of its interfaces are limited:
-      // Q_c - dt/dx [(A+dQ - F)_{c-1/2} + (A-dQ + F)_{c+1/2}]
-      R qout[K][M], Fl[M], FK[M];
-      limit1d<RP, R, LIMC>(C, order, Wm, W[0], s[0], K > 1 ? W[1] : Wp, dtdx, Fl);
-#pragma unroll
-      for (int k = 0; k < M; ++k) FK[k] = __shfl_down_sync(FULL, Fl[k], 1);
-#pragma unroll
-      for (int c = 1; c < K; ++c) {
-        R Fr[M];
-        limit1d<RP, R, LIMC>(C, order, W[c - 1], W[c], s[c], c + 1 < K ? W[c + 1] : Wp, dtdx, Fr);
-#pragma unroll
-        for (int k = 0; k < M; ++k) {
-          qout[c - 1][k] = qa[c - 1][k] - dtdx * ((ap[c - 1][k] - Fl[k]) + (am[c][k] + Fr[k]));
-          Fl[k] = Fr[k];
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < M; ++k)
-        qout[K - 1][k] = qa[K - 1][k] - dtdx * ((ap[K - 1][k] - Fl[k]) + (amK[k] + FK[k]));
+      R qout[K][M];
+      unit1d<RP, R, K, FAST>(C, order, dtdx, lk, qa, aa, lane, nx + 1 - g0, qout, smax);
 
       // non-finite results: FP32 folds them into one sum of v * 0 (NaN for
       // a NaN or an infinity, else 0) tested once per item; FP64 tests each
@@ -614,6 +757,154 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 && RP::M <= 2) ? (K >= 8 ?
 }
 
 // ---------------------------------------------------------------------------
+// Several attempts of one small 1D grid in one launch: a single thread-block
+// cluster takes the grid's warp units, with one hardware cluster barrier per
+// attempt.  Each block stores its largest speed and flags into every block's
+// shared memory (distributed shared memory), and after the barrier each block
+// runs the controller on its own copy of the control block: the same values,
+// so the same dt and buffer index everywhere.  The reports alternate between
+// two sets, since a block may be one attempt ahead of a slower one.  The
+// states alternate in global memory, read past L1 (ld.cg), since other blocks
+// of this launch wrote them.  What an attempt costs is then one L2 round trip,
+// the unit's arithmetic, a barrier and the controller, in place of a launch
+// and a chain of some eight L2 round trips.  The arithmetic is unit1d, so the
+// results are those of single attempts.
+// ---------------------------------------------------------------------------
+template <class RP, typename R, int K, bool FAST>
+__global__ void __launch_bounds__(kCluster1dThreads)
+    classic1d_cluster_kernel(const Member* __restrict__ members, const MConsts<R> C, int attempts) {
+  namespace cg = cooperative_groups;
+  constexpr int M = RP::M, MA = RP::MA, MAS = MA > 0 ? MA : 1;
+  constexpr int WC = 30 * K, NW = kCluster1dThreads / 32;
+  constexpr int kWords = sizeof(DevCtl) / 8;
+  static_assert(sizeof(DevCtl) % 8 == 0, "the control block moves as 8-byte words");
+  __shared__ DevCtl s_ctl;                   // the block's copy of the control block
+  __shared__ unsigned long long s_rep[2][16];  // every block's largest speed ...
+  __shared__ unsigned s_repbad[2][16];         // ... and flags, by attempt parity
+  __shared__ unsigned long long s_max;       // of this block's warps
+  __shared__ unsigned s_bad;
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank(), nblk = (int)cl.num_blocks();
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const Member& mb = members[0];
+  DevCtl* ctl = mb.ctl;
+  for (int i = threadIdx.x; i < kWords; i += kCluster1dThreads)
+    ((unsigned long long*)&s_ctl)[i] = ((const unsigned long long*)ctl)[i];
+  if (threadIdx.x == 0) {
+    s_max = 0ull;
+    s_bad = 0u;
+  }
+  const int nx = mb.nx;
+  R* const buf0 = (R*)mb.q[0];  // the classic 1D step alternates between two
+  R* const buf1 = (R*)mb.q[1];
+  const R* __restrict__ aux = (const R*)mb.aux;
+  const int order = FAST ? 2 : C.order;
+  const int units = (nx + WC - 1) / WC;
+  const bool aligned = (M == 1 || ((size_t)nx * sizeof(R)) % 16 == 0) &&
+                       ((((size_t)buf0) | ((size_t)buf1)) & 15) == 0;
+  cl.sync();  // every block has started and has its copy
+  for (int at = 0; at < attempts; ++at) {
+    if (s_ctl.done) break;  // the same in every block
+    const int par = at & 1;
+    const R* q = s_ctl.cur ? buf1 : buf0;
+    R* qo = s_ctl.cur ? buf0 : buf1;
+    const R dtdx = dt_over_dx<R>(&s_ctl, 0);
+    LinK<R> lk{};
+    if constexpr (is_linear_rp<RP, R>::value) Lin<RP, R>::consts(C, 0, dtdx, lk);
+    R smax = R(0);
+    int bad = 0;
+    for (int u = rank + nblk * w; u < units; u += nblk * NW) {
+      const int g0 = u * WC + (lane - 1) * K;
+      const bool inside = g0 >= 0 && g0 + K <= nx;
+      R qa[K][M], aa[K][MAS];
+#pragma unroll
+      for (int k = 0; k < M; ++k) {
+        R v[K];
+        if (inside && aligned) {
+          VecIO<R, K>::load_l2(q + (size_t)k * nx + g0, v);
+        } else {
+#pragma unroll
+          for (int c = 0; c < K; ++c) {
+            // ghost cells by remap; cells beyond the ghost layer clamped into it
+            int flip, inflow;
+            const int j =
+                bc_map(max(-2, min(g0 + c, nx + 1)), nx, C.bc_lo[0], C.bc_hi[0], flip, inflow);
+            v[c] = inflow ? C.inflow[k] : __ldcg(q + (size_t)k * nx + j);
+            if (flip && k == RP::WALL_X) v[c] = -v[c];
+          }
+        }
+#pragma unroll
+        for (int c = 0; c < K; ++c) qa[c][k] = v[c];
+      }
+      if constexpr (MA > 0) {
+#pragma unroll
+        for (int c = 0; c < K; ++c)
+          load_aux<MA, R>(C, aux, nx, 1, max(-2, min(g0 + c, nx + 1)), 0, aa[c]);
+      }
+      R qout[K][M];
+      R sm = R(0);
+      unit1d<RP, R, K, FAST>(C, order, dtdx, lk, qa, aa, lane, nx + 1 - g0, qout, sm);
+      smax = nanmax(smax, sm);
+      if (lane >= 1 && lane <= 30) {
+#pragma unroll
+        for (int k = 0; k < M; ++k) {
+          R v[K];
+#pragma unroll
+          for (int c = 0; c < K; ++c) {
+            v[c] = qout[c][k];
+            if (g0 + c < nx) bad |= not_finite(v[c]);
+          }
+          if (inside && aligned) {
+            VecIO<R, K>::store(qo + (size_t)k * nx + g0, v);
+          } else {
+#pragma unroll
+            for (int c = 0; c < K; ++c)
+              if (g0 + c < nx) qo[(size_t)k * nx + g0 + c] = v[c];
+          }
+        }
+      }
+    }
+    // the block's largest speed (as bit patterns: not negative, a NaN wins) and
+    // flags, reported to every block
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      smax = nanmax(smax, __shfl_xor_sync(0xffffffffu, smax, o));
+      bad |= __shfl_xor_sync(0xffffffffu, bad, o);
+    }
+    if (lane == 0) {
+      const double d = (double)smax;
+      if (d != 0.0) atomicMax(&s_max, (unsigned long long)__double_as_longlong(d));
+      if (bad) atomicOr(&s_bad, 1u);
+    }
+    __syncthreads();
+    if (threadIdx.x < nblk) {
+      *cl.map_shared_rank(&s_rep[par][rank], threadIdx.x) = s_max;
+      *cl.map_shared_rank(&s_repbad[par][rank], threadIdx.x) = s_bad;
+    }
+    cl.sync();
+    if (w == 0) {
+      unsigned long long m = lane < nblk ? s_rep[par][lane] : 0ull;
+      unsigned bd = lane < nblk ? s_repbad[par][lane] : 0u;
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) {
+        const unsigned long long x = __shfl_xor_sync(0xffffffffu, m, o);
+        m = x > m ? x : m;
+        bd |= __shfl_xor_sync(0xffffffffu, bd, o);
+      }
+      if (lane == 0) {
+        s_max = 0ull;
+        s_bad = 0u;
+        control_step(&s_ctl, s_ctl.dt * __longlong_as_double((long long)m) / s_ctl.dx[0], bd);
+      }
+    }
+    __syncthreads();
+  }
+  if (rank == 0)
+    for (int i = threadIdx.x; i < kWords; i += kCluster1dThreads)
+      ((unsigned long long*)ctl)[i] = ((const unsigned long long*)&s_ctl)[i];
+}
+
+// ---------------------------------------------------------------------------
 // 2D unsplit step.  A block of BW threads owns a strip of BW-4 interior
 // columns and walks down H interior rows of it.  Thread l holds column
 // c = c0 - 2 + l.  Per row R it solves the x-interface (c, R) and the
@@ -674,6 +965,7 @@ __global__ void __launch_bounds__(BW)
   __shared__ int s_done, s_cur, s_nbuf;
   __shared__ R s_k[3];  // dt/dx, dt/dy, dt^2/(2 dx dy)
   const int l = threadIdx.x;
+  pdl_enter();
 
   for (int it = blockIdx.x; it < ntiles_total; it += gridDim.x) {
     const Tile tl = tiles ? tiles[it] : Tile{0, it};

@@ -129,6 +129,7 @@ __global__ void __launch_bounds__(32 * kXSweepLines, sizeof(R) == 4 ? 2 : 1)
   __shared__ int s_done, s_cur, s_nbuf;
   const Member& mb = members[0];
   DevCtl* ctl = mb.ctl;
+  pdl_enter();
   if (threadIdx.x < 3) LS::consts(C, threadIdx.x, dt_over_dx<R>(ctl, threadIdx.x), K[threadIdx.x]);
   if (threadIdx.x == 32) {
     s_done = ctl->done;

@@ -126,6 +126,16 @@ __device__ __forceinline__ int bc_map(int i, int n, int bclo, int bchi, int& fli
   return i;
 }
 
+// Entry of a kernel launched as a programmatic dependent of the previous
+// launch on its stream: wait until that launch has completed and its memory is
+// visible, then let the next launch begin (its blocks wait here in turn), so
+// that launch latency overlaps this kernel.  For a launch without the
+// attribute both return at once.
+__device__ __forceinline__ void pdl_enter() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // dt / dx_d of the current attempt.  FP64: the quotient; FP32: one multiply by
 // the stored 1/dx before the rounding (an FP64 division at each block's start
 // takes some 600 cycles on the FP64 pipe).
@@ -251,23 +261,8 @@ __device__ __forceinline__ int clip_final(double t, double t_end, double& dt) {
 // reject (keep Q^n, shrink dt by cfl_desired/nu) above cfl_max, otherwise
 // accept (advance t, rotate buffers); then choose dt_next = dt*cfl_desired/nu,
 // bounded by dt_max and clipped to land on t_end.
-static __device__ __noinline__ void run_controller(DevCtl* c) {
-  if (c->dry) {
-    c->smax[0] = 0ull;
-    c->smax[1] = 0ull;
-    c->smax[2] = 0ull;
-    c->bad = 0u;
-    __threadfence();
-    c->arrive = 0u;
-    return;
-  }
-  const unsigned bad = atomicOr(&c->bad, 0u);
+static __device__ __forceinline__ void control_step(DevCtl* c, double nu, unsigned bad) {
   const double dt = c->dt;
-  double nu = dt * __longlong_as_double((long long)atomicOr(&c->smax[0], 0ull)) / c->dx[0];
-  for (int d = 1; d < c->ndim; ++d) {
-    const double v = dt * __longlong_as_double((long long)atomicOr(&c->smax[d], 0ull)) / c->dx[d];
-    nu = (nu >= v || isnan(nu)) ? nu : v;
-  }
   c->accepted = 0;
   if (bad || isnan(nu)) {
     // bit 1: a non-finite value; bit 2: a bounded wait gave up
@@ -301,12 +296,35 @@ static __device__ __noinline__ void run_controller(DevCtl* c) {
     c->dt = nd;
     if (c->t >= c->t_end || c->steps >= c->max_steps) c->done = 1;
   }
-  c->smax[0] = 0ull;
-  c->smax[1] = 0ull;
-  c->smax[2] = 0ull;
-  c->bad = 0u;
-  __threadfence();
-  c->arrive = 0u;
+}
+// ... on the control block in global memory, from the speeds and flags that
+// the attempt's blocks folded into it.  The block comes in one round trip past
+// L1 (independent 16-byte loads; the attempt's atomics are in the L2 by the
+// arrivals' fences or the launch boundary), the decision runs on registers, and
+// the block goes back whole: nothing else of the attempt touches it any more.
+static __device__ __noinline__ void run_controller(DevCtl* c) {
+  static_assert(sizeof(DevCtl) % 8 == 0, "the control block moves as 8-byte words");
+  constexpr int kW = sizeof(DevCtl) / 8;
+  union {
+    unsigned long long w[kW];
+    DevCtl v;
+  } u;
+#pragma unroll
+  for (int i = 0; i < kW; ++i) u.w[i] = __ldcg((const unsigned long long*)c + i);
+  if (!u.v.dry) {
+    const double dt = u.v.dt;
+    double nu = dt * __longlong_as_double((long long)u.v.smax[0]) / u.v.dx[0];
+    for (int d = 1; d < u.v.ndim; ++d) {
+      const double v = dt * __longlong_as_double((long long)u.v.smax[d]) / u.v.dx[d];
+      nu = (nu >= v || isnan(nu)) ? nu : v;
+    }
+    control_step(&u.v, nu, u.v.bad);
+  }
+  u.v.smax[0] = u.v.smax[1] = u.v.smax[2] = 0ull;
+  u.v.bad = 0u;
+  u.v.arrive = 0u;
+#pragma unroll
+  for (int i = 0; i < kW; ++i) ((unsigned long long*)c)[i] = u.w[i];
 }
 
 // Reduce two per-thread maxima and a bad flag over the block (in the working

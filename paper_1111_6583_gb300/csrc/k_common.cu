@@ -184,6 +184,7 @@ size_t faces_work_bytes(int nd, int nx, int ny, int m, int prec) {
 }
 
 __global__ void controllers_kernel(const Member* __restrict__ members, int n) {
+  pdl_enter();
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k < n) {
     DevCtl* c = members[k].ctl;
@@ -192,8 +193,7 @@ __global__ void controllers_kernel(const Member* __restrict__ members, int n) {
 }
 
 cudaError_t launch_controllers(const Member* members, int n, cudaStream_t st) {
-  controllers_kernel<<<(n + 127) / 128, 128, 0, st>>>(members, n);
-  return cudaGetLastError();
+  return launch_pdl(controllers_kernel, (n + 127) / 128, 128, st, members, n);
 }
 
 cudaError_t launch_source_mark(const Member* members, int n, cudaStream_t st) {

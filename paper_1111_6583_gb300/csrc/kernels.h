@@ -32,11 +32,28 @@ struct LaunchArgs {
   size_t work3_bytes;
   const StageOp* stage_op; // SharpClaw: explicit stage (host pointer) or null
   int sweep;               // 2D classic: 0 unsplit, 1 / 2 the x / y sweeps of a split step
+  int attempts;            // 1D: attempts of one launch (KernelSet::multi1d)
   int nmembers;            // members of the table (1D classic runs their controllers after)
   int src_phase;           // source step: 0 Godunov (dt after an accepted step), 1 Strang
                            // pre (dt/2 of the attempt, slot cur -> qpre), 2 Strang post
                            // (dt/2 after an accepted step)
 };
+
+// Launch as a programmatic dependent of the previous launch on the stream (the
+// kernel begins with pdl_enter)
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kern)(P...), int grid, int threads, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
 
 // stage tables of the SharpClaw time integrators
 int stage_table(int integrator, const StageOp** ops);  // returns the number of stages
@@ -54,7 +71,9 @@ struct KernelSet {
   int max_bw;              // 2D classic: widest block whose static shared memory fits
   int tx64, tx128;         // 2D classic: columns of a tile at either width
   int tx64_walk, tx128_walk;  // ... of the row walk, for systems that also run it (else 0)
+  int linear;              // constant-coefficient linear system (strength form)
   int reg_kernel;          // 2D classic: register-resident kernel (chunks of 2 rows pay)
+  launch_fn multi1d;       // 1D classic: several attempts of one small grid (one member)
   int (*blocks3)(int nx, int ny, int nz);  // 3D: blocks of an attempt (they count the arrivals)
   int sharp_shapes;        // 2D SharpClaw WENO5: bit i set when tile kSharpShapes2[i]
                            // fits in a block's shared memory
@@ -85,6 +104,19 @@ inline int classic1d_tiles(int nx, int prec, int ma) {
 // 1D classic work modes (LaunchArgs::h): a warp takes a whole tile, or one
 // unit of it; any other value: whole tiles when they fill every resident warp
 constexpr int kWork1dTiles = 1, kWork1dUnits = 2;
+// Several attempts in one launch of one cluster (at most 16 blocks, 64 SM
+// sub-partitions): grids whose warp units (30 K cells) give each sub-partition
+// little enough to do that the whole GPU's launch and round trips cost more.
+// us/step, cluster against single launches: acoustics FP64 2000 cells 6.5 / 10.1
+// (12.7 before the strength form), 4000 7.0 / 9.8, 8000 10.4 / 9.8; FP32 2000
+// 5.7 / 9.8, 64,000 7.4 / 9.8, 128,000 9.7 / 10.6, 256,000 13.1 / 10.4; Euler
+// FP64 2000 17.8 / 21.5, 4000 23.2 / 22.0, FP32 8000 9.1 / 11.3, 16,000 11.1 /
+// 11.0; elasticity FP32 4000 4.8 / 8.9.
+constexpr int kCluster1dThreads = 256;
+inline bool cluster1d_fits(long long nx, int prec, int ma, bool linear) {
+  const long long units = (nx + 30 * classic1d_K(prec, ma) - 1) / (30 * classic1d_K(prec, ma));
+  return units <= (linear ? (prec == 0 ? 96 : 512) : 64);
+}
 constexpr int kSharpTX2 = 16, kSharpTY2 = 8;  // 2D SharpClaw tile (default)
 constexpr int kSharpTX1 = 128;                // 1D SharpClaw tile
 // shared memory one block may hold on the device (227 KB)

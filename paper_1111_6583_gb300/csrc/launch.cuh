@@ -218,11 +218,10 @@ struct Launchers {
     if constexpr (ND == 3) {
       const long long nx = a.n3[0], ny = a.n3[1], nz = a.n3[2];
       const Layout3 L = layout3d((int)nx, (int)ny, (int)nz, sizeof(R) == 8 ? 0 : 1);
-      const unsigned grid = (unsigned)classic3d_blocks(L);
+      const int grid = classic3d_blocks(L);
       if (C.lim == CLAW_LIM_MC && C.order == 2 && C.transverse == 2)
-        classic3d_kernel<RP, R, true><<<grid, 32 * kXSweepLines, 0, a.stream>>>(a.members, C, L);
-      else
-        classic3d_kernel<RP, R, false><<<grid, 32 * kXSweepLines, 0, a.stream>>>(a.members, C, L);
+        return launch_pdl(classic3d_kernel<RP, R, true>, grid, 32 * kXSweepLines, a.stream, a.members, C, L);
+      return launch_pdl(classic3d_kernel<RP, R, false>, grid, 32 * kXSweepLines, a.stream, a.members, C, L);
       return cudaGetLastError();
     } else if constexpr (medium_kernel<RP, ND>()) {
       const bool fast = C.lim == CLAW_LIM_MC && C.order == 2 && C.transverse == 2 && a.sweep == 0;
@@ -255,8 +254,53 @@ struct Launchers {
   template <class K>
   static cudaError_t reg2d(K kern, const LaunchArgs& a, const MConsts<R>& C) {
     const int threads = 32 * reg_tile(sizeof(R) == 8 ? 0 : 1, a.bw).warps;
-    kern<<<launch_grid(a.ntiles_total), threads, 0, a.stream>>>(a.members, a.tiles, C, a.h, a.sweep);
-    return cudaGetLastError();
+    return launch_pdl(kern, launch_grid(a.ntiles_total), threads, a.stream, a.members, a.tiles, C, a.h, a.sweep);
+  }
+  // a.attempts attempts of one grid in one launch of one cluster (1D)
+  static cudaError_t multi1d(const LaunchArgs& a) {
+    if constexpr (ND == 1) {
+      const MConsts<R>& C = *(const MConsts<R>*)a.consts;
+      constexpr int K = classic1d_K(sizeof(R) == 8 ? 0 : 1, RP::MA);
+      if (sizeof(R) == 4 && C.lim == CLAW_LIM_MC && C.order == 2)
+        return cluster1d<classic1d_cluster_kernel<RP, R, K, sizeof(R) == 4>>(a, C);
+      return cluster1d<classic1d_cluster_kernel<RP, R, K, false>>(a, C);
+    } else {
+      (void)a;
+      return cudaErrorNotSupported;
+    }
+  }
+  template <auto Kern>
+  static cudaError_t cluster1d(const LaunchArgs& a, const MConsts<R>& C) {
+    // sixteen blocks where the device can place such a cluster, else the
+    // portable eight (asked once per kernel)
+    static const unsigned blocks = [] {
+      cudaFuncSetAttribute(Kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      cudaLaunchConfig_t c = {};
+      c.gridDim = dim3(16);
+      c.blockDim = dim3(kCluster1dThreads);
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = 16;
+      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+      c.attrs = at;
+      c.numAttrs = 1;
+      int n = 0;
+      const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, Kern, &c);
+      if (e != cudaSuccess) cudaGetLastError();
+      return e == cudaSuccess && n >= 1 ? 16u : 8u;
+    }();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(kCluster1dThreads);
+    cfg.stream = a.stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = blocks;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, Kern, a.members, C, a.attempts);
+    return e != cudaSuccess ? e : cudaGetLastError();
   }
   template <bool FAST>
   static cudaError_t roe2d(const LaunchArgs& a, const MConsts<R>& C) {
@@ -264,9 +308,8 @@ struct Launchers {
       constexpr int prec = sizeof(R) == 8 ? 0 : 1;
       using V = typename std::conditional<sizeof(R) == 8, double, F2>::type;
       auto go = [&](auto kern, int threads) {
-        kern<<<launch_grid(a.ntiles_total), threads, 0, a.stream>>>(a.members, a.tiles, C, a.h,
-                                                                   a.sweep);
-        return cudaGetLastError();
+        return launch_pdl(kern, launch_grid(a.ntiles_total), threads, a.stream, a.members, a.tiles, C, a.h,
+                          a.sweep);
       };
       constexpr int w64 = roe_tile(prec, 64).warps, w128 = roe_tile(prec, 128).warps;
       if (a.bw == 128) return go(roe2d_kernel<RP, V, w128, FAST>, 32 * w128);
@@ -288,25 +331,12 @@ struct Launchers {
       const long long cap = (long long)persistent_grid<kt>(kClassic1dThreads, 1 << 30) * NW;
       const bool whole =
           a.h == kWork1dTiles || (a.h != kWork1dUnits && a.ntiles_total >= cap);
-      if (whole)
-        kt<<<persistent_grid<kt>(kClassic1dThreads, (a.ntiles_total + NW - 1) / NW),
-             kClassic1dThreads, 0, a.stream>>>(a.members, a.tiles, a.ntiles_total, C);
-      else {
-        // single units (small grids, where launch latency is the step's
-        // cost): a programmatic dependent launch on the previous attempt
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)persistent_grid<ku>(kClassic1dThreads, a.ntiles_total));
-        cfg.blockDim = dim3(kClassic1dThreads);
-        cfg.dynamicSmemBytes = 0;
-        cfg.stream = a.stream;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        const cudaError_t el = cudaLaunchKernelEx(&cfg, ku, a.members, a.tiles, a.ntiles_total, C);
-        if (el != cudaSuccess) return el;
-      }
+      const cudaError_t el =
+          whole ? launch_pdl(kt, persistent_grid<kt>(kClassic1dThreads, (a.ntiles_total + NW - 1) / NW),
+                             kClassic1dThreads, a.stream, a.members, a.tiles, a.ntiles_total, C)
+                : launch_pdl(ku, persistent_grid<ku>(kClassic1dThreads, a.ntiles_total),
+                             kClassic1dThreads, a.stream, a.members, a.tiles, a.ntiles_total, C);
+      if (el != cudaSuccess) return el;
       const cudaError_t e = cudaGetLastError();
       if (e != cudaSuccess || !whole) return e;  // single units run their controllers
       return launch_controllers(a.members, a.nmembers > 0 ? a.nmembers : 1, a.stream);
@@ -332,15 +362,13 @@ struct Launchers {
                          (!is_roe2d<RP>::value || (sizeof(R) == 4 && !FAST))) {
       if constexpr (classic2d_fits<RP, R>(128)) {
         if (a.bw == 128) {
-          classic2d_kernel<RP, R, 128, FAST><<<launch_grid(a.ntiles_total), 128, 0, a.stream>>>(
-              a.members, a.tiles, a.ntiles_total, C, a.h, a.sweep);
-          return cudaGetLastError();
+          return launch_pdl(classic2d_kernel<RP, R, 128, FAST>, launch_grid(a.ntiles_total), 128,
+                            a.stream, a.members, a.tiles, a.ntiles_total, C, a.h, a.sweep);
         }
       }
       if (a.bw != 64) return cudaErrorInvalidValue;
-      classic2d_kernel<RP, R, 64, FAST><<<launch_grid(a.ntiles_total), 64, 0, a.stream>>>(
-          a.members, a.tiles, a.ntiles_total, C, a.h, a.sweep);
-      return cudaGetLastError();
+      return launch_pdl(classic2d_kernel<RP, R, 64, FAST>, launch_grid(a.ntiles_total), 64, a.stream,
+                        a.members, a.tiles, a.ntiles_total, C, a.h, a.sweep);
     } else {
       (void)a;
       (void)C;
@@ -384,10 +412,8 @@ struct Launchers {
   template <int RW>
   static cudaError_t sharp_launch(const LaunchArgs& a, const MConsts<R>& C, const StageOp& op) {
     if constexpr (ND == 1) {
-      sharp_stage_kernel<RP, R, 1, kSharpTX1, 1, RW>
-          <<<launch_grid(a.ntiles_total), kSharpTX1, 0, a.stream>>>(a.members, a.tiles,
-                                                                 a.ntiles_total, C, op);
-      return cudaSuccess;
+      return launch_pdl(sharp_stage_kernel<RP, R, 1, kSharpTX1, 1, RW>, launch_grid(a.ntiles_total),
+                        kSharpTX1, a.stream, a.members, a.tiles, a.ntiles_total, C, op);
     } else if constexpr (ND == 2) {
       int tx, ty;
       sharp2d_shape(a.bw, a.h, tx, ty);
@@ -408,10 +434,8 @@ struct Launchers {
   template <int TX, int TY, int RW>
   static cudaError_t sharp2d(const LaunchArgs& a, const MConsts<R>& C, const StageOp& op) {
     if constexpr (sharp_smem_bytes<RP, R, 2, TX, TY, RW>() <= kSmemPerBlock) {
-      sharp_stage_kernel<RP, R, 2, TX, TY, RW>
-          <<<launch_grid(a.ntiles_total), TX * TY, 0, a.stream>>>(a.members, a.tiles,
-                                                                 a.ntiles_total, C, op);
-      return cudaSuccess;
+      return launch_pdl(sharp_stage_kernel<RP, R, 2, TX, TY, RW>, launch_grid(a.ntiles_total), TX * TY,
+                        a.stream, a.members, a.tiles, a.ntiles_total, C, op);
     } else {
       (void)a;
       (void)C;
@@ -460,6 +484,8 @@ KernelSet make_set(bool has_char) {
   k.maxspeed = &Launchers<RP, R, ND>::maxspeed;
   k.source = &Launchers<RP, R, ND>::source;
   k.blocks3 = &Launchers<RP, R, ND>::blocks3;
+  k.linear = is_linear_rp<RP, R>::value ? 1 : 0;
+  k.multi1d = ND == 1 ? &Launchers<RP, R, ND>::multi1d : nullptr;
   k.max_bw = classic2d_fits<RP, R>(128) ? 128 : 64;
   constexpr bool roe = ND == 2 && is_roe2d<RP>::value;
   k.reg_kernel = ND == 2 && (is_linear_rp<RP, R>::value || medium_kernel<RP, ND>() || roe);

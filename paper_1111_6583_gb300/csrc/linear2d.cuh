@@ -79,6 +79,7 @@ __global__ void __launch_bounds__(32 * reg_tile(sizeof(R) == 8 ? 0 : 1, BW).warp
   const Tile tl = tiles ? tiles[blockIdx.x] : Tile{0, (int)blockIdx.x};
   const Member& mb = members[tl.member];
   DevCtl* ctl = mb.ctl;
+  pdl_enter();  // (the tables above do not change between attempts)
   if (ctl->done) return;  // the whole block
   const int lane = threadIdx.x & 31;
   if (threadIdx.x < 2) {

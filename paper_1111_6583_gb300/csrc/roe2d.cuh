@@ -347,6 +347,7 @@ __global__ void __launch_bounds__(32 * NWB, VecOf<V>::N == 1 ? 0 : 12 / NWB)
   const Tile tl = tiles ? tiles[blockIdx.x] : Tile{0, (int)blockIdx.x};
   const Member& mb = members[tl.member];
   DevCtl* ctl = mb.ctl;
+  pdl_enter();  // (the tables above do not change between attempts)
   if (ctl->done) return;  // the whole block
   const int lane = threadIdx.x & 31;
   const R lx = dt_over_dx<R>(ctl, 0), ly = dt_over_dx<R>(ctl, 1);

@@ -223,6 +223,7 @@ __global__ void __launch_bounds__(TX * TY, sharp_minb<R, TX, TY, RW>())
     }
   }
 
+  pdl_enter();
   for (int it = blockIdx.x; it < ntiles_total; it += gridDim.x) {
     const Tile tl = tiles ? tiles[it] : Tile{0, it};
     const Member& mb = members[tl.member];
