@@ -216,25 +216,19 @@ __device__ __forceinline__ void limit1d(const MConsts<R>& C, int order,
     return;
   }
   R dot[MW], nrm[MW];
-  constexpr int KS = strength_k<RP, 0>();
 #pragma unroll
   for (int p = 0; p < MW; ++p) {
     // upwind neighbour: left for a right-going wave
     const bool right = signed_waves<RP>::value ? p != 0 : sc[p] > R(0);
-    if constexpr (KS >= 0) {
-      dot[p] = right ? Wl[p][KS] : Wr[p][KS];
-      nrm[p] = Wc[p][KS];
-    } else {
-      R d = R(0), n2 = R(0);
+    R d = R(0), n2 = R(0);
 #pragma unroll
-      for (int k = 0; k < M; ++k) {
-        const R up = right ? Wl[p][k] : Wr[p][k];
-        d += up * Wc[p][k];
-        n2 += Wc[p][k] * Wc[p][k];
-      }
-      dot[p] = d;
-      nrm[p] = n2;
+    for (int k = 0; k < M; ++k) {
+      const R up = right ? Wl[p][k] : Wr[p][k];
+      d += up * Wc[p][k];
+      n2 += Wc[p][k] * Wc[p][k];
     }
+    dot[p] = d;
+    nrm[p] = n2;
   }
   correction<RP, R, 0, LIMC>(C, Wc, sc, dot, nrm, dtdx, F);
 }
@@ -932,21 +926,19 @@ __device__ __forceinline__ void solve_cells(const MConsts<R>& C, const R (&ql)[R
 // sweep: 0 the unsplit step (Q^n in slot 0 -> slot 1, runs the controller);
 // dimensional splitting (Godunov) as two launches: 1 the x sweeps (slot 0 ->
 // slot 1), 2 the y sweeps (slot 1 -> slot 2, runs the controller).
-// FAST: the MC limiter, second order and transverse mode 2 fixed at compile
-// time (the launcher takes it for FP32 methods with those settings)
-template <class RP, typename R, int BW, bool FAST = false>
+// For Euler and, in FP32 with van Leer's limiter, shallow water (the other
+// systems and settings have their own kernels: linear2d.cuh, medium2d.cuh,
+// roe2d.cuh).
+template <class RP, typename R, int BW>
 __global__ void __launch_bounds__(BW)
     classic2d_kernel(const Member* __restrict__ members, const Tile* __restrict__ tiles,
                      int ntiles_total, const MConsts<R> C, int H, int sweep) {
   constexpr int M = RP::M, MW = RP::MW, NC = RP::NCTX;
-  constexpr int LIMC = FAST ? CLAW_LIM_MC : -1;
-  const int order = FAST ? 2 : C.order;
-  const int transverse = FAST ? 2 : C.transverse;
+  const int order = C.order;
+  const int transverse = C.transverse;
   constexpr int NP = RP::NPC > 0 ? RP::NPC : 1;
   using NZX = typename RP::template NZ<0>;
   using NZY = typename RP::template NZ<1>;
-  // limiter ratios from wave strengths where the solver has them
-  constexpr int KSX = strength_k<RP, 0>(), KSY = strength_k<RP, 1>();
   constexpr int TX = BW - 4;
   // neighbour contributions: systems of up to three fields publish the raw
   // vectors (the receiver multiplies and adds them, saving the sender's pass
@@ -975,7 +967,7 @@ __global__ void __launch_bounds__(BW)
       s_done = ctl->done;
       s_k[0] = dt_over_dx<R>(ctl, 0);
       s_k[1] = dt_over_dx<R>(ctl, 1);
-      s_k[2] = R(0.5) * s_k[0] * s_k[1];
+      s_k[2] = half_dt2_over_dxdy<R>(ctl);
       s_cur = ctl->cur;
       s_nbuf = ctl->nbuf;
     }
@@ -1058,21 +1050,15 @@ __global__ void __launch_bounds__(BW)
         solve_cells<RP, 1, R, NP>(C, qm1, qc, pm1, pcc, nW, ns, nam, nap, nx_);
 #pragma unroll
         for (int p = 0; p < MW; ++p) {
-          if constexpr (KSY >= 0) {
-            // wave strengths: the new interface's strength serves as its
-            // "norm" and as the upper neighbour's term of interface Rw-1
-            nnrm[p] = ndot[p] = nW[p][KSY];
-          } else {
-            R a = R(0), b = R(0);
+          R a = R(0), b = R(0);
 #pragma unroll
-            for (int k = 0; k < M; ++k) {
-              if (!NZY::f(p, k)) continue;
-              a += nW[p][k] * nW[p][k];
-              b += nW[p][k] * yW[p][k];
-            }
-            nnrm[p] = a;
-            ndot[p] = b;
+          for (int k = 0; k < M; ++k) {
+            if (!NZY::f(p, k)) continue;
+            a += nW[p][k] * nW[p][k];
+            b += nW[p][k] * yW[p][k];
           }
+          nnrm[p] = a;
+          ndot[p] = b;
         }
         if (col_in && Rw >= r0 && Rw <= rend + 1) {
 #pragma unroll
@@ -1117,22 +1103,17 @@ __global__ void __launch_bounds__(BW)
 #pragma unroll
           for (int p = 0; p < MW; ++p) {
             const int lu = gt0(xs[p]) ? l - 1 : l + 1;
-            if constexpr (KSX >= 0) {
-              dot[p] = xws[p][KSX][lu];
-              nrm[p] = xW[p][KSX];
-            } else {
-              R a = R(0), b = R(0);
+            R a = R(0), b = R(0);
 #pragma unroll
-              for (int k = 0; k < M; ++k) {
-                if (!NZX::f(p, k)) continue;
-                b += xws[p][k][lu] * xW[p][k];
-                a += xW[p][k] * xW[p][k];
-              }
-              dot[p] = b;
-              nrm[p] = a;
+            for (int k = 0; k < M; ++k) {
+              if (!NZX::f(p, k)) continue;
+              b += xws[p][k][lu] * xW[p][k];
+              a += xW[p][k] * xW[p][k];
             }
+            dot[p] = b;
+            nrm[p] = a;
           }
-          correction<RP, R, 0, LIMC>(C, xW, xs, dot, nrm, dtdx, F);
+          correction<RP, R, 0>(C, xW, xs, dot, nrm, dtdx, F);
         } else {
 #pragma unroll
           for (int k = 0; k < M; ++k) F[k] = R(0);
@@ -1183,7 +1164,7 @@ __global__ void __launch_bounds__(BW)
           R dot[MW];
 #pragma unroll
           for (int p = 0; p < MW; ++p) dot[p] = gt0(ys[p]) ? ydot[p] : ndot[p];
-          correction<RP, R, 1, LIMC>(C, yW, ys, dot, ynrm, dtdy, G);
+          correction<RP, R, 1>(C, yW, ys, dot, ynrm, dtdy, G);
         } else {
 #pragma unroll
           for (int k = 0; k < M; ++k) G[k] = R(0);
@@ -1301,14 +1282,8 @@ __global__ void __launch_bounds__(BW)
 #pragma unroll
         for (int p = 0; p < MW; ++p) {
           ys[p] = ns[p];
-          if constexpr (KSY >= 0) {
-            // the lower neighbour's strength of the next interface to limit
-            ydot[p] = ynrm[p];
-            ynrm[p] = nnrm[p];
-          } else {
-            ynrm[p] = nnrm[p];
-            ydot[p] = ndot[p];
-          }
+          ynrm[p] = nnrm[p];
+          ydot[p] = ndot[p];
 #pragma unroll
           for (int k = 0; k < M; ++k) yW[p][k] = nW[p][k];
         }

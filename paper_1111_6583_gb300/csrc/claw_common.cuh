@@ -144,6 +144,13 @@ __device__ __forceinline__ R dt_over_dx(const DevCtl* c, int d) {
   if constexpr (sizeof(R) == 4) return (R)(c->dt * c->idx[d]);
   else return c->dt / c->dx[d];
 }
+// dt^2 / (2 dx dy), rounded once (the product of two quotients rounded to FP32
+// would be off by up to three roundings in every transverse term)
+template <typename R>
+__device__ __forceinline__ R half_dt2_over_dxdy(const DevCtl* c) {
+  if constexpr (sizeof(R) == 4) return (R)(0.5 * (c->dt * c->idx[0]) * (c->dt * c->idx[1]));
+  else return 0.5 * (c->dt / c->dx[0]) * (c->dt / c->dx[1]);
+}
 
 // Load cell (c, r) of a field-major array q[M][ny][nx] with ghost remap.  In
 // 2D the value of a corner ghost is the y-rule applied to the x-rule value of

@@ -220,9 +220,10 @@ struct Launchers {
       const Layout3 L = layout3d((int)nx, (int)ny, (int)nz, sizeof(R) == 8 ? 0 : 1);
       const int grid = classic3d_blocks(L);
       if (C.lim == CLAW_LIM_MC && C.order == 2 && C.transverse == 2)
-        return launch_pdl(classic3d_kernel<RP, R, true>, grid, 32 * kXSweepLines, a.stream, a.members, C, L);
-      return launch_pdl(classic3d_kernel<RP, R, false>, grid, 32 * kXSweepLines, a.stream, a.members, C, L);
-      return cudaGetLastError();
+        return launch_pdl(classic3d_kernel<RP, R, true>, grid, 32 * kXSweepLines, a.stream,
+                          a.members, C, L);
+      return launch_pdl(classic3d_kernel<RP, R, false>, grid, 32 * kXSweepLines, a.stream,
+                        a.members, C, L);
     } else if constexpr (medium_kernel<RP, ND>()) {
       const bool fast = C.lim == CLAW_LIM_MC && C.order == 2 && C.transverse == 2 && a.sweep == 0;
       if (a.bw != 64 && a.bw != 128) return cudaErrorInvalidValue;
@@ -240,15 +241,11 @@ struct Launchers {
         return classic1d<true>(a, C);
       return classic1d<false>(a, C);
     } else {
-      // systems of up to three fields: with more, the two block widths of the
-      // fixed-settings form were seen to round differently, and every tile
-      // shape must give the same bits
-      if ((sizeof(R) == 4 || is_linear_rp<RP, R>::value || is_roe2d<RP>::value) && RP::M <= 3 && C.lim == CLAW_LIM_MC && C.order == 2 &&
-          C.transverse == 2 && a.sweep == 0)
+      if ((is_linear_rp<RP, R>::value || is_roe2d<RP>::value) && C.lim == CLAW_LIM_MC &&
+          C.order == 2 && C.transverse == 2 && a.sweep == 0)
         return classic2d<true>(a, C);
       return classic2d<false>(a, C);
     }
-    return cudaGetLastError();
   }
   // one launch of a register-resident 2D kernel (a block per tile)
   template <class K>
@@ -346,6 +343,8 @@ struct Launchers {
       return cudaErrorNotSupported;
     }
   }
+  // FAST (strength forms only, whose bits do not depend on it): the common
+  // settings fixed at compile time
   template <bool FAST>
   static cudaError_t classic2d(const LaunchArgs& a, const MConsts<R>& C) {
     if constexpr (ND == 2 && is_roe2d<RP>::value) {
@@ -358,16 +357,16 @@ struct Launchers {
       if (a.bw == 128) return reg2d(linear2d_kernel<RP, R, 128, FAST>, a, C);
       if (a.bw == 64) return reg2d(linear2d_kernel<RP, R, 64, FAST>, a, C);
       return cudaErrorInvalidValue;
-    } else if constexpr (ND == 2 && RP::MA == 0 && (!FAST || (sizeof(R) == 4 && RP::M <= 3)) &&
-                         (!is_roe2d<RP>::value || (sizeof(R) == 4 && !FAST))) {
+    } else if constexpr (ND == 2 && RP::MA == 0 && !FAST &&
+                         (!is_roe2d<RP>::value || sizeof(R) == 4)) {
       if constexpr (classic2d_fits<RP, R>(128)) {
         if (a.bw == 128) {
-          return launch_pdl(classic2d_kernel<RP, R, 128, FAST>, launch_grid(a.ntiles_total), 128,
+          return launch_pdl(classic2d_kernel<RP, R, 128>, launch_grid(a.ntiles_total), 128,
                             a.stream, a.members, a.tiles, a.ntiles_total, C, a.h, a.sweep);
         }
       }
       if (a.bw != 64) return cudaErrorInvalidValue;
-      return launch_pdl(classic2d_kernel<RP, R, 64, FAST>, launch_grid(a.ntiles_total), 64, a.stream,
+      return launch_pdl(classic2d_kernel<RP, R, 64>, launch_grid(a.ntiles_total), 64, a.stream,
                         a.members, a.tiles, a.ntiles_total, C, a.h, a.sweep);
     } else {
       (void)a;
