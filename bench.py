@@ -47,6 +47,9 @@ L2_FLUSH_BYTES = 512 << 20
 #   medium constants it re-derives at every interface (c = sqrt(K/rho): one
 #   division and one square root; Z = rho c and 2 Z twice: three products),
 #   which the kernel takes as constants.
+# The strength-form kernels take the same step with fewer operations than
+# these counts of the wave-vector form, so a fraction of an ALU peak by them
+# can exceed one.
 # Bytes: one read and one write of the conserved fields (plus aux reads).
 SW2D_FLOPS_PER_CELL = 825.0
 EULER2D_WENO5_FLOPS_PER_CELL_STAGE = 3032.4
@@ -55,12 +58,8 @@ ACOU1D_FLOPS_PER_CELL = 90.0
 SW2D_BYTES_PER_CELL = {"fp64": 48.0, "fp32": 24.0}
 ELAST1D_BYTES_PER_CELL = {"fp64": 48.0, "fp32": 24.0}  # q read+write, aux read
 ACOU1D_BYTES_PER_CELL = {"fp64": 32.0, "fp32": 16.0}   # q read+write
-# 3D acoustics (4 fields, w bytes per value), per cell and step: the x sweep
-# reads the state and stores five face records (6 m w); the y and z sweeps
-# read the state, store two records and reduce into three, a read and a write
-# each at the DRAM (9 m w each); the update reads the state and nine records
-# and writes the state (11 m w): 35 m w in all
-ACOU3D_BYTES_PER_CELL = {"fp32": 35 * 4 * 4, "fp64": 35 * 4 * 8}
+# 3D acoustics (4 fields): the step reads and writes the state once
+ACOU3D_BYTES_PER_CELL = {"fp32": 2 * 4 * 4, "fp64": 2 * 4 * 8}
 # ALU peaks from unit counts and clocks (for comparison with the measured FMA
 # rate the roofline uses): 152 SMs x 2.07 GHz x 2 FLOP per FMA x FMA lanes per
 # SM per clock (FP64: 2; FP32: 128)
@@ -69,8 +68,8 @@ FP32_PEAK_DERIVED_TFLOPS = 152 * 2.07e9 * 2 * 128 / 1e12
 
 
 TRAFFIC_RECORD = os.path.join(ROOT, "profiles", "traffic_classic2d_sw_fp64_1024.json")
-KERNEL_SOURCES = ["claw_common.cuh", "riemann.cuh", "classic.cuh", "launch.cuh", "kernels.h",
-                  "k_sw.cu"]
+KERNEL_SOURCES = ["claw_common.cuh", "riemann.cuh", "linear.cuh", "linear2d.cuh", "vec.cuh",
+                  "roe2d.cuh", "launch.cuh", "kernels.h", "k_sw.cu"]
 
 
 def kernel_sha():
@@ -98,7 +97,7 @@ def recorded_traffic(tile):
 def record_traffic(csv_path, tile):
     """Write the traffic record from an ncu --csv launch list of the bench
     command (metrics dram__bytes_read.sum, dram__bytes_write.sum; the last
-    four classic2d launches of `--case sw2d1024` are its four steps; ncu
+    four step launches of `--case sw2d1024` are its four steps; ncu
     flushes the caches before each launch it captures, so these are the
     bytes of a launch that starts with a cold L2, as the timed steps do)."""
     import csv
@@ -113,11 +112,11 @@ def record_traffic(csv_path, tile):
     timed = list(by.values())[-4:]
     b = sum(v["dram__bytes_read.sum"] + v["dram__bytes_write.sum"] for v in timed) / len(timed)
     t = "%d,%d" % tuple(tile)
-    rec = {"kernel": "classic2d_kernel<RpSW<double,2>>", "workload": "dam break 1024x1024 FP64",
+    rec = {"kernel": "roe2d_kernel<RpSW<double,2>>", "workload": "dam break 1024x1024 FP64",
            "tile": list(tile), "dram_bytes_per_launch": b, "sources_sha256": kernel_sha(),
            "command": "python bench.py --case sw2d1024 --tile %s > plain.log 2>&1 && "
                       "ncu --metrics gpu__time_duration.sum,dram__bytes_read.sum,"
-                      "dram__bytes_write.sum --clock-control none -k regex:classic2d --csv "
+                      "dram__bytes_write.sum --clock-control none -k regex:roe2d --csv "
                       "--log-file traffic_sw2d.csv python bench.py --case sw2d1024 "
                       "--tile %s" % (t, t)}
     json.dump(rec, open(TRAFFIC_RECORD, "w"), indent=1)
@@ -504,8 +503,7 @@ def bench_axisym(prec, steps, warmup, nx=1280, ny=320, dim_split=0, source_split
 
 def bench_acoustics_vc(prec, steps, warmup, n=1024):
     """2D acoustics in a heterogeneous medium on a stretched grid (capacity):
-    classic with full transverse corrections on the per-face path (two face
-    sweeps + the update per step)."""
+    classic with full transverse corrections (one fused launch per step)."""
     import torch
     from paper_1111_6583_gb300 import claw
     from paper_1111_6583_gb300 import workloads as wl
@@ -522,13 +520,13 @@ def bench_acoustics_vc(prec, steps, warmup, n=1024):
     avg = sum(ms) / len(ms)
     return {"value": n * n * len(ms) / (sum(ms) * 1e-3), "unit": UNIT, "ms_per_step": avg,
             "workload": "2D acoustics, varying medium + capacity %dx%d, classic full "
-                        "transverse (per-face path), %s" % (n, n, prec.upper())}
+                        "transverse, %s" % (n, n, prec.upper())}
 
 
 def bench_acoustics_table1(prec, steps, warmup, nd, n):
-    """The paper's Table 1 acoustics system, constant medium: 2D on n^2 (row
-    kernel, autotuned tiles) or 3D on n^3 (a memset, three face sweeps with
-    transverse and double-transverse terms, the update)."""
+    """The paper's Table 1 acoustics system, constant medium: 2D on n^2
+    (autotuned tiles) or 3D on n^3 with transverse and double-transverse terms
+    (one fused launch per step)."""
     import torch
     from paper_1111_6583_gb300 import claw
     from paper_1111_6583_gb300 import workloads as wl
@@ -1150,7 +1148,7 @@ def main():
         ex["axisym_shock_bubble"] = ax
         at = {"2d_" + p: bench_acoustics_table1(p, 20, 3, 2, 1024) for p in ("fp64", "fp32")}
         at.update({"3d_" + p: bench_acoustics_table1(p, 5, 3, 3, 256) for p in ("fp64", "fp32")})
-        # 3D: algorithmic bytes per cell and step over the four launches
+        # 3D: the state read and written once per step
         g3 = ACOU3D_BYTES_PER_CELL["fp32"] * 256 ** 3 / (at["3d_fp32"]["ms_per_step"] * 1e-3)
         at["3d_fp32"]["hbm_gbs"] = g3 / 1e9
         at["3d_fp32"]["hbm_frac"] = g3 / 1e9 / hbm

@@ -221,11 +221,11 @@ claw_status claw_solver_destroy(claw_solver* s);
 /* launch per step over a table of tiles (each grid keeps its own t, dt).  */
 /* ---------------------------------------------------------------------- */
 
-/* grids[n]: one per member (same ndim and method; 1D, 2D or 3D).  Row-kernel
- * methods run one fused launch per step over all members' tiles; methods on
- * the per-face classic path (a capacity field, or 2D varying-medium
- * acoustics) and 3D grids (the face sweeps and update of Sec. 2's 3D
- * algorithm) run their kernels member by member inside each attempt. */
+/* grids[n]: one per member (same ndim and method; 1D, 2D or 3D).  Tiled methods
+ * (1D and 2D, varying-medium acoustics with or without a capacity among
+ * them) run one fused launch per step over all members' tiles; methods on
+ * the per-face classic path (a capacity field with another system) and 3D
+ * grids run their kernels member by member inside each attempt. */
 claw_status claw_batch_create(const claw_method* m, const claw_grid* grids, int n, void* stream,
                               claw_batch** out);
 /* q[k], aux[k]: device pointers of member k (caller-owned); t_end[k]. */
@@ -264,14 +264,14 @@ typedef struct {
  * work buffers, aux, control blocks; with a Strang-split source one more
  * state buffer; on the per-face classic path its face arrays).  max_slots
  * bounds concurrent requests.  Classic 1D/2D and SharpClaw methods, with or
- * without a source term; on the per-face path (a capacity field, or 2D
- * varying-medium acoustics) the kernels run request by request. */
+ * without a source term; on the per-face path (a capacity field with a system other
+ * than 2D varying-medium acoustics) the kernels run request by request. */
 claw_status claw_server_create(const claw_method* m, size_t hbm_budget_bytes, int max_slots,
                                void* stream, claw_server** out);
 /* The same for grids of ndim dimensions (1, 2 or 3; claw_server_create takes
  * 2 when num_eqn is the 2D system's field count, else 1).  3D requests run
- * the classic face sweeps and update request by request (Sec. 2's 3D
- * algorithm with transverse and double-transverse terms). */
+ * the classic step request by request (Sec. 2's 3D algorithm with transverse
+ * and double-transverse terms). */
 claw_status claw_server_create_nd(const claw_method* m, int ndim, size_t hbm_budget_bytes,
                                   int max_slots, void* stream, claw_server** out);
 /* Submit one solve: grid, initial state (host memory, the method's precision

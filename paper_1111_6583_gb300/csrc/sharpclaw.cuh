@@ -117,7 +117,7 @@ __device__ __forceinline__ void weno5_fields(const R (&w)[M][5], R eps, R (&um)[
   }
 }
 
-// WENO of order 2 RW - 1 (7 .. 17; WENO5 takes weno5_pair): left-biased value at the right edge of cell
+// WENO of order 2 RW - 1 (7 .. 17; WENO5 takes weno5_diff): left-biased value at the right edge of cell
 // v[o + RW - 1] from v[o .. o + 2 RW - 2] (REV: the mirrored stencil, value at
 // the left edge of cell v[o + RW], read from v[o + 2 RW - 1] downwards).
 template <int RW, bool REV, typename R, int NV>
