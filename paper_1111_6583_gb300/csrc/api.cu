@@ -631,7 +631,13 @@ cudaError_t build_graph(claw_solver* s, int k) {
 // Time candidate (bw, h) shapes of the 2D classic kernel on the bound state
 // with a dry control block (attempts leave t, dt and the state untouched) and
 // keep the fastest.
-cudaError_t autotune(claw_solver* s) {
+// brief: a few shapes only, where an attempt is so short that timing all of
+// them would cost a new solver more than its first steps (2D varying-medium
+// acoustics on its first evolve; claw_solver_tune times all).
+// 16 steps of a new solver, all shapes -> these: FP32 1024^2 4.03 -> 1.45 ms,
+// 200 x 181 1.98 -> 0.61; FP64 301 x 280 7.2 -> 2.3, 100 x 90 5.0 -> 1.1; the
+// steps themselves as fast or within 5 % (FP32 1024^2 0.69 -> 0.71).
+cudaError_t autotune(claw_solver* s, bool brief) {
   if (s->m.scheme == CLAW_CLASSIC && s->nd == 1 && !s->faces) {
     // 1D: how warps take work (whole tiles or single units)
     int bw = s->bw, h = s->h;
@@ -683,9 +689,13 @@ cudaError_t autotune(claw_solver* s) {
   for (int bw : bws) {
     if (bw > s->ks.max_bw) continue;
     for (int h : {8, 16, 32, 64, 128})
-      if (h <= 2 * ny) cand.push_back({bw, h});
+      if (h <= 2 * ny && !brief) cand.push_back({bw, h});
     for (int k = 1; k <= 8; ++k) {
       if (nsm <= 0) break;
+      // brief: one or two tiles of two FP64 warps per pair of sub-partitions;
+      // two FP32 one-warp tiles per sub-partition (and one, of the wider)
+      const bool few = s->prec == 0 ? k == 2 || k == 4 : k == 8 || (k == 4 && bw == s->ks.max_bw);
+      if (brief && !few) continue;
       int h = s->ks.reg_kernel ? 2 : 4;
       while (h < ny && tiles_of(s->ks, s->m.scheme, 2, s->prec, nx, ny, bw, h) > k * nsm) ++h;
       // (heights that cut the rows into as many chunks are the same tiles)
@@ -924,7 +934,7 @@ claw_status claw_solver_tune(claw_solver* s, int mode, int* bw, int* h) {
   if (!s || !s->bound) return fail(s, "solver not bound");
   if (mode == 0) {
     SCK(enter(s));
-    SCK(autotune(s));
+    SCK(autotune(s, false));
     SCK(leave(s));
   } else {
     if (s->m.scheme == CLAW_CLASSIC && s->nd == 1 && h &&
@@ -997,7 +1007,7 @@ claw_status claw_evolve_to_time(claw_solver* s, double t_end, int64_t max_steps,
                                 claw_step_info* info) {
   if (!s || !s->bound) return fail(s, "solver not bound");
   SCK(enter(s));
-  if (!s->tuned && !multi1d(s)) SCK(autotune(s));
+  if (!s->tuned && !multi1d(s)) SCK(autotune(s, s->m.rp == CLAW_RP_ACOUSTICS_VC));
   SCK(launch_set_t_end(s->d_ctl, 1, t_end, (long long)max_steps, s->st));
   const int GK = 16;
   if (use_graph && s->gk != GK) SCK(build_graph(s, GK));
